@@ -466,30 +466,6 @@ __global__ void __launch_bounds__(kThreads) mlp_train_seq_kernel(MlpDev w, const
     backward_tile(sm, ns, 1.f / static_cast<float>(B), parts + static_cast<size_t>(blockIdx.x) * (NPARAM + 1));
 }
 
-// Predicted next slopes of every subaperture from the 4 newest rows of a history
-// ring: s_pred = s_k + sigma * y (x block then y block).
-__global__ void __launch_bounds__(kThreads) mlp_predict_kernel(MlpDev w, const float* __restrict__ ring,
-                                                               int kpad, int head, int nv,
-                                                               const int* __restrict__ nbr, float sigma,
-                                                               float* __restrict__ s_pred) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    const int s0 = blockIdx.x * TM;
-    const int ns = min(TM, nv - s0);
-    load_weights(sm, w);
-    const float* rows[4];
-    for (int lag = 0; lag < 4; ++lag) rows[lag] = ring + static_cast<size_t>((head - lag + 4) & 3) * kpad;
-    gather_pairs(sm, false, nbr, nv, 1.f / sigma, [&](int si) { return si < ns ? s0 + si : -1; },
-                 [&](int, int lag) { return rows[lag]; });
-    __syncthreads();
-    forward_tile(sm, false);
-    const float* Y = reinterpret_cast<const float*>(sm + Smem::Y);
-    for (int q = threadIdx.x; q < ns * NO; q += kThreads) {
-        const int s = q / NO, o = q - s * NO;
-        const int idx = o * nv + s0 + s;
-        s_pred[idx] = __fmaf_rn(sigma, Y[q], rows[0][idx]);
-    }
-}
-
 // Sum of the CTA partials in a fixed pairwise order, then (when lr > 0) one Adam step
 // on the FP32 master weights and a refresh of the BF16 copies.  grad_out (optional)
 // receives the summed gradient; loss_out (optional) the loss sum / (2B).
@@ -548,8 +524,7 @@ cudaError_t mlp_configure() {
     cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_train_seq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_predict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    return e;
+    return e == cudaSuccess ? mlp_predict_configure() : e;
 }
 
 cudaError_t mlp_launch_refresh(const MlpDev& w, cudaStream_t st) {
@@ -573,14 +548,6 @@ cudaError_t mlp_launch_train_seq(const MlpDev& w, const float* S, int n_frames, 
 
 cudaError_t mlp_launch_forward(const MlpDev& w, const float* X, int B, float* Y, cudaStream_t st) {
     mlp_forward_kernel<<<(B + TM - 1) / TM, kThreads, Smem::TOTAL, st>>>(w, X, B, Y);
-    return cudaGetLastError();
-}
-
-cudaError_t mlp_launch_predict(const MlpDev& w, const float* ring, int kpad, int head, int nv,
-                               const int* nbr, float sigma, float* s_pred, cudaStream_t st) {
-    if (nv == 0) return cudaSuccess;
-    mlp_predict_kernel<<<(nv + TM - 1) / TM, kThreads, Smem::TOTAL, st>>>(w, ring, kpad, head, nv, nbr,
-                                                                         sigma, s_pred);
     return cudaGetLastError();
 }
 

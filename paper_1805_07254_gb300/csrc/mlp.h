@@ -25,8 +25,11 @@ cudaError_t mlp_launch_train_seq(const MlpDev& w, const float* S, int n_frames, 
                                  const int* nbr, const int2* samples, int B, float inv_sigma,
                                  float* parts, cudaStream_t st);
 cudaError_t mlp_launch_forward(const MlpDev& w, const float* X, int B, float* Y, cudaStream_t st);
-cudaError_t mlp_launch_predict(const MlpDev& w, const float* ring, int kpad, int head, int nv,
-                               const int* nbr, float sigma, float* s_pred, cudaStream_t st);
+// Predictions of frames k0 .. k0 + nk - 1 of a slope sequence S [][2 nv] (features of
+// rows k .. k-3) into rows k + 1 of out, in one launch (mlp_predict.cu).
+cudaError_t mlp_predict_configure();
+cudaError_t mlp_launch_predict(const MlpDev& w, const float* S, float* out, int k0, int nk, int nv, const int* nbr,
+                               float sigma, int sms, cudaStream_t st);
 // Sum the partials; lr > 0 also applies Adam step `step` (from 1).
 cudaError_t mlp_launch_update(const MlpDev& w, const float* parts, int nparts, int B, float lr,
                               float beta1, float beta2, float eps, int step, float* grad_out,

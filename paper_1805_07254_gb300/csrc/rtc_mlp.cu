@@ -18,6 +18,7 @@ struct rtc_mlp {
     int* d_nbr = nullptr;        // [nv][25] neighbour table (rtc_mlp_set_geometry)
     int nv = 0;
     int step = 0;                // Adam steps taken
+    int sms = 1;                 // streaming multiprocessors of the device
 };
 
 namespace {
@@ -121,6 +122,7 @@ int rtc_mlp_create(int32_t device, rtc_mlp** out) {
     if (mlp_configure() != cudaSuccess) return mfail(RTC_EDEVICE, "cannot configure the MLP kernels");
     rtc_mlp* m = new rtc_mlp();
     m->device = device;
+    cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, device);
     const int rc = mlp_alloc(m->w);
     if (rc != RTC_OK) {
         mlp_free(m->w);
@@ -245,13 +247,14 @@ extern "C" int rtc_mlp_predict_seq(rtc_mlp* m, const float* d_S, int32_t n_frame
     if (!m || !d_S || !d_out || n_frames < 0 || !(sigma > 0.f)) return mfail(RTC_EINVAL, "bad arguments");
     if (!m->d_nbr && m->nv > 0) return mfail(RTC_ESTATE, "rtc_mlp_set_geometry first");
     Dev d(m->device);
-    const size_t row = 2 * static_cast<size_t>(m->nv);
+    const size_t len = 2 * static_cast<size_t>(m->nv) * n_frames * sizeof(float);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    for (int k = 3; k <= n_frames - 2; ++k) {
-        // rows k-3 .. k of the sequence play the history ring with the newest in slot 3
-        if (mlp_launch_predict(m->w, d_S + (k - 3) * row, static_cast<int>(row), 3, m->nv, m->d_nbr,
-                               sigma, d_out + (k + 1) * row, st) != cudaSuccess)
+    // every frame in one launch; an output that overlaps the sequence is fed back frame
+    // by frame, so there each frame is a launch of its own
+    const uintptr_t a = reinterpret_cast<uintptr_t>(d_S), b = reinterpret_cast<uintptr_t>(d_out);
+    const int nk = n_frames - 4, step = a < b + len && b < a + len ? 1 : nk;
+    for (int k = 3; k < 3 + nk; k += step)
+        if (mlp_launch_predict(m->w, d_S, d_out, k, step, m->nv, m->d_nbr, sigma, m->sms, st) != cudaSuccess)
             return mfail(RTC_EDEVICE, "prediction launch failed");
-    }
     return RTC_OK;
 }
