@@ -1,0 +1,31 @@
+// Programmatic dependent launch: a kernel launched with launch_pdl may be scheduled
+// while the stream's previous kernel still runs (if that kernel lets it, or drains).
+// Its blocks call pdl_wait() before they read or write anything another kernel may
+// touch: it returns once the previous kernel has completed and its writes are visible.
+// A kernel calls pdl_launch_dependents() only after its own pdl_wait(), so that
+// whatever precedes it in the stream is complete before its successor starts.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <utility>
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(std::forward<A>(args))...);
+}

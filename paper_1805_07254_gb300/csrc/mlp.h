@@ -15,16 +15,22 @@ struct MlpDev {
     __nv_bfloat16* w2_bf16;      // [64][64] BF16 copy of W2
 };
 
-size_t mlp_smem_bytes();
-cudaError_t mlp_configure();
+// Samples of a training tile; floats from one block's partial gradient to the next
+// (RTC_MLP_NPARAMS, the loss sum, padding to the update kernel's 64).
+constexpr int kMlpTile = 32;
+constexpr int kMlpPartPitch = 17216;
+// Blocks (and so partials) of a batch: one per tile up to the SM count.
+__host__ __device__ inline int mlp_tiles(int B) { return B / kMlpTile + (B % kMlpTile != 0); }
+inline int mlp_blocks(int B, int sms) { return mlp_tiles(B) < sms ? mlp_tiles(B) : sms; }
+
 cudaError_t mlp_launch_refresh(const MlpDev& w, cudaStream_t st);
-// CTA partial gradients of a batch: parts [ceil(B/64)][RTC_MLP_NPARAMS + 1] (last = loss sum).
-cudaError_t mlp_launch_train(const MlpDev& w, const float* X, const float* T, int B, float* parts,
+// Partial gradients of a batch: parts [blocks][kMlpPartPitch].
+cudaError_t mlp_launch_train(const MlpDev& w, const float* X, const float* T, int B, float* parts, int blocks,
                              cudaStream_t st);
 cudaError_t mlp_launch_train_seq(const MlpDev& w, const float* S, int n_frames, int nv,
                                  const int* nbr, const int2* samples, int B, float inv_sigma,
-                                 float* parts, cudaStream_t st);
-cudaError_t mlp_launch_forward(const MlpDev& w, const float* X, int B, float* Y, cudaStream_t st);
+                                 float* parts, int blocks, cudaStream_t st);
+cudaError_t mlp_launch_forward(const MlpDev& w, const float* X, int B, float* Y, int sms, cudaStream_t st);
 // Predictions of frames k0 .. k0 + nk - 1 of a slope sequence S [][2 nv] (features of
 // rows k .. k-3) into rows k + 1 of out, in one launch (mlp_predict.cu).
 cudaError_t mlp_predict_configure();

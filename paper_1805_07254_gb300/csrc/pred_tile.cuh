@@ -102,13 +102,16 @@ __device__ __forceinline__ float relu_nan(float z) {
     asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(z));
     return y;
 }
-__device__ __forceinline__ float gelu(float z) {
-    const float a = fminf(fabsf(z), kGeluMax);
+// erfc(a / sqrt 2) for 0 <= a <= kGeluMax.
+__device__ __forceinline__ float gelu_erfc(float a) {
     float q = kGelu.c[kGeluTerms - 1];
 #pragma unroll
     for (int k = kGeluTerms - 2; k >= 0; --k) q = __fmaf_rn(q, a, kGelu.c[k]);
-    const float e = ex2(__fmul_rn(a, q));
-    return __fmaf_rn(-0.5f, __fmul_rn(a, e), relu_nan(z));
+    return ex2(__fmul_rn(a, q));
+}
+__device__ __forceinline__ float gelu(float z) {
+    const float a = fminf(fabsf(z), kGeluMax);
+    return __fmaf_rn(-0.5f, __fmul_rn(a, gelu_erfc(a)), relu_nan(z));
 }
 
 // Two GELUs with packed FP32 arithmetic: the same bits as gelu() of each.

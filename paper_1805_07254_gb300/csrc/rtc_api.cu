@@ -702,7 +702,6 @@ int rtc_load_predictor(rtc_handle* h, const float* params, int64_t n, float sigm
     DeviceScope ds(h->cfg.device);
     RTC_CUDA(h, cudaStreamSynchronize(h->stream));
     free_predictor(h);
-    RTC_CUDA(h, mlp_configure());
     h->pred = new MlpDev();
     if (mlp_alloc(*h->pred) != RTC_OK) {
         free_predictor(h);

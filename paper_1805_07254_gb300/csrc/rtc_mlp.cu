@@ -13,7 +13,7 @@
 struct rtc_mlp {
     int device = 0;
     MlpDev w{};
-    float* parts = nullptr;      // [nparts_cap][RTC_MLP_NPARAMS + 1] CTA partials
+    float* parts = nullptr;      // [nparts_cap][kMlpPartPitch] block partials
     int nparts_cap = 0;
     int* d_nbr = nullptr;        // [nv][25] neighbour table (rtc_mlp_set_geometry)
     int nv = 0;
@@ -22,8 +22,6 @@ struct rtc_mlp {
 };
 
 namespace {
-
-constexpr int kTile = 64;        // samples per CTA of the MLP kernels
 
 int mfail(int code, const char* msg) {
     rtc_set_global_error(msg);
@@ -43,12 +41,12 @@ struct Dev {
 };
 
 int ensure_parts(rtc_mlp* m, int B) {
-    const int need = (B + kTile - 1) / kTile;
+    const int need = mlp_blocks(B, m->sms);
     if (need <= m->nparts_cap) return RTC_OK;
     if (m->parts) cudaFree(m->parts);
     m->parts = nullptr;
     m->nparts_cap = 0;
-    if (cudaMalloc(&m->parts, static_cast<size_t>(need) * (RTC_MLP_NPARAMS + 1) * sizeof(float)) != cudaSuccess)
+    if (cudaMalloc(&m->parts, static_cast<size_t>(need) * kMlpPartPitch * sizeof(float)) != cudaSuccess)
         return mfail(RTC_ENOMEM, "cannot allocate the gradient partials");
     m->nparts_cap = need;
     return RTC_OK;
@@ -119,7 +117,7 @@ int rtc_mlp_create(int32_t device, rtc_mlp** out) {
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev)
         return mfail(RTC_EINVAL, "device not available");
     Dev d(device);
-    if (mlp_configure() != cudaSuccess) return mfail(RTC_EDEVICE, "cannot configure the MLP kernels");
+    if (mlp_predict_configure() != cudaSuccess) return mfail(RTC_EDEVICE, "cannot configure the MLP kernels");
     rtc_mlp* m = new rtc_mlp();
     m->device = device;
     cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, device);
@@ -187,7 +185,7 @@ int rtc_mlp_forward(rtc_mlp* m, const float* d_X, int32_t B, float* d_Y, void* s
     if (!m || B < 0 || (B > 0 && (!d_X || !d_Y))) return mfail(RTC_EINVAL, "bad arguments");
     if (B == 0) return RTC_OK;
     Dev d(m->device);
-    if (mlp_launch_forward(m->w, d_X, B, d_Y, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+    if (mlp_launch_forward(m->w, d_X, B, d_Y, m->sms, static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return mfail(RTC_EDEVICE, "forward launch failed");
     return RTC_OK;
 }
@@ -199,8 +197,8 @@ int rtc_mlp_gradient(rtc_mlp* m, const float* d_X, const float* d_T, int32_t B, 
     int rc = ensure_parts(m, B);
     if (rc != RTC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, st) != cudaSuccess ||
-        mlp_launch_update(m->w, m->parts, (B + kTile - 1) / kTile, B, 0.f, 0.9f, 0.999f, 1e-8f, 1,
+    if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, mlp_blocks(B, m->sms), st) != cudaSuccess ||
+        mlp_launch_update(m->w, m->parts, mlp_blocks(B, m->sms), B, 0.f, 0.9f, 0.999f, 1e-8f, 1,
                           d_grad, d_loss, st) != cudaSuccess)
         return mfail(RTC_EDEVICE, "gradient launch failed");
     return RTC_OK;
@@ -214,8 +212,8 @@ int rtc_mlp_train_step(rtc_mlp* m, const float* d_X, const float* d_T, int32_t B
     if (rc != RTC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     m->step += 1;
-    if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, st) != cudaSuccess ||
-        mlp_launch_update(m->w, m->parts, (B + kTile - 1) / kTile, B, lr, 0.9f, 0.999f, 1e-8f,
+    if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, mlp_blocks(B, m->sms), st) != cudaSuccess ||
+        mlp_launch_update(m->w, m->parts, mlp_blocks(B, m->sms), B, lr, 0.9f, 0.999f, 1e-8f,
                           m->step, nullptr, d_loss, st) != cudaSuccess)
         return mfail(RTC_EDEVICE, "training launch failed");
     return RTC_OK;
@@ -233,8 +231,8 @@ int rtc_mlp_train_seq(rtc_mlp* m, const float* d_S, int32_t n_frames, const int3
     m->step += 1;
     if (mlp_launch_train_seq(m->w, d_S, n_frames, m->nv, m->d_nbr,
                              reinterpret_cast<const int2*>(d_samples), B, 1.f / sigma, m->parts,
-                             st) != cudaSuccess ||
-        mlp_launch_update(m->w, m->parts, (B + kTile - 1) / kTile, B, lr, 0.9f, 0.999f, 1e-8f,
+                             mlp_blocks(B, m->sms), st) != cudaSuccess ||
+        mlp_launch_update(m->w, m->parts, mlp_blocks(B, m->sms), B, lr, 0.9f, 0.999f, 1e-8f,
                           m->step, nullptr, d_loss, st) != cudaSuccess)
         return mfail(RTC_EDEVICE, "training launch failed");
     return RTC_OK;
