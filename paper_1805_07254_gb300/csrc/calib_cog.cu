@@ -1,39 +1,53 @@
 // Stand-alone pixel stage: calibration, centre of gravity and slope packing for
-// every valid subaperture of every WFS (Sec. 2.1, Fig. 3 (a)-(b)); one warp per
-// subaperture (see pixel.cuh).  The fused frame kernel runs the same device code.
+// every valid subaperture of every WFS (Sec. 2.1, Fig. 3 (a)-(b)); a half-warp per
+// subaperture, as in the fused frame kernel, which runs the same device code
+// (pixel.cuh).
+//
+// An ELT frame is 4 MB in and 32 KB out: two dependent rounds of loads (position,
+// pixels), not bandwidth.  So the stage's time in a run of frames is mostly launch and
+// drain, and the launches overlap (programmatic dependent launch): a block fetches its
+// subapertures' positions and calibration data while the previous kernel drains, and
+// waits for it only before it reads pixels.  The slopes go straight into the caller's
+// buffer as well as the resident one.  Measured, ELT, frame after frame: 3.0 us a frame
+// on the GPU (4.4 us with the caller's Python) against 10.2 us for a warp per
+// subaperture in a plain launch and a device copy of the slopes after it.
 
+#include "launch.cuh"
 #include "pixel.cuh"
 
 namespace {
 
-constexpr int kWarpsPerBlock = kCalibThreads / 32;
+constexpr int kPerBlock = kCalibThreads / 16;
 
 template <int NPX>
 __global__ void __launch_bounds__(kCalibThreads) calib_cog_kernel(rtc_pixel::PixelArgs p) {
-    const int gw = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (gw >= p.n_valid * p.n_wfs) return;
-    rtc_pixel::subap_slopes<NPX, rtc_pixel::kPixelReadOnly, 32>(p, p.frame, p.s, gw, true,
-                                                                threadIdx.x & 31);
+    const int gi = blockIdx.x * kPerBlock + (threadIdx.x >> 4);
+    const bool valid = gi < p.n_valid * p.n_wfs;
+    const int2 pos = rtc_pixel::subap_pos(p, gi, valid);
+    rtc_pixel::subap_slopes_at<NPX, rtc_pixel::kPixelReadOnly, 16>(
+        p, p.frame, p.s, gi, valid, threadIdx.x & 31, pos, rtc_pixel::NoHook(), []() {
+            pdl_wait();
+            pdl_launch_dependents();
+        });
 }
 
 }  // namespace
 
-rtc_pixel::PixelArgs pixel_args(const rtc_handle* h, const uint16_t* d_frame, float* d_s) {
-    return rtc_pixel::PixelArgs{d_frame,    h->side,     h->cfg.npx, h->n_valid, h->cfg.n_wfs,
-                                h->d_rc,    h->d_dark,   h->d_gainmap, h->thr_mode, h->thr, d_s};
+rtc_pixel::PixelArgs pixel_args(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2) {
+    return rtc_pixel::PixelArgs{d_frame,   h->side,      h->cfg.npx,  h->n_valid, h->cfg.n_wfs, h->d_rc,
+                                h->d_dark, h->d_gainmap, h->thr_mode, h->thr,     d_s,          d_s2};
 }
 
-cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s,
+cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2,
                              cudaStream_t st) {
-    const int warps = h->n_valid * h->cfg.n_wfs;
-    if (warps == 0) return cudaSuccess;
-    const int blocks = (warps + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    const rtc_pixel::PixelArgs p = pixel_args(h, d_frame, d_s);
+    const int n = h->n_valid * h->cfg.n_wfs;
+    if (n == 0) return cudaSuccess;
+    const dim3 grid((n + kPerBlock - 1) / kPerBlock), block(kCalibThreads);
+    const rtc_pixel::PixelArgs p = pixel_args(h, d_frame, d_s, d_s2);
     switch (h->cfg.npx) {
-        case 8: calib_cog_kernel<8><<<blocks, kCalibThreads, 0, st>>>(p); break;
-        case 10: calib_cog_kernel<10><<<blocks, kCalibThreads, 0, st>>>(p); break;
-        case 16: calib_cog_kernel<16><<<blocks, kCalibThreads, 0, st>>>(p); break;
-        default: calib_cog_kernel<0><<<blocks, kCalibThreads, 0, st>>>(p); break;
+        case 8: return launch_pdl(calib_cog_kernel<8>, grid, block, 0, st, p);
+        case 10: return launch_pdl(calib_cog_kernel<10>, grid, block, 0, st, p);
+        case 16: return launch_pdl(calib_cog_kernel<16>, grid, block, 0, st, p);
+        default: return launch_pdl(calib_cog_kernel<0>, grid, block, 0, st, p);
     }
-    return cudaGetLastError();
 }

@@ -263,11 +263,11 @@ cudaError_t launch_pred(const rtc_handle* h, const Launch& L, rtc_pixel::PixelAr
 
 template <int DT>
 cudaError_t launch_dt(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float* d_s_meas,
-                      int head, cudaStream_t st, FrameHost* fhp) {
+                      int head, cudaStream_t st, FrameHost* fhp, float* d_s2) {
     const bool pred = d_s_meas != nullptr;
     const Launch L = plan_launch(h, pred ? rtc_pred::kSmemBytes : 0);
     if (!L.ok) return cudaErrorInvalidValue;
-    const rtc_pixel::PixelArgs px = pixel_args(h, d_frame, pred ? d_s_meas : h->d_s);
+    const rtc_pixel::PixelArgs px = pixel_args(h, d_frame, pred ? d_s_meas : h->d_s, d_s2);
     const Args g = make_args(h, h->d_s, d_dm_out, L);
     // the block count may change between launches (e.g. a server slot limits it), so
     // each target is the running total of expected arrivals, not launches x blocks
@@ -346,14 +346,14 @@ rtc_pred::PredArgs pred_args(const rtc_handle* h) {
 }
 
 cudaError_t launch_frame(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float* d_s_meas,
-                         int head, cudaStream_t st, FrameHost* fh) {
+                         int head, cudaStream_t st, FrameHost* fh, float* d_s2) {
     if (h->kpad == 0) return launch_decay(h, d_dm_out, st);
     switch (h->store) {
-        case RTC_F32: return launch_dt<RTC_F32>(h, d_frame, d_dm_out, d_s_meas, head, st, fh);
-        case RTC_BF16: return launch_dt<RTC_BF16>(h, d_frame, d_dm_out, d_s_meas, head, st, fh);
-        case RTC_F16: return launch_dt<RTC_F16>(h, d_frame, d_dm_out, d_s_meas, head, st, fh);
-        case RTC_FP8_E4M3: return launch_dt<RTC_FP8_E4M3>(h, d_frame, d_dm_out, d_s_meas, head, st, fh);
-        case RTC_INT8: return launch_dt<RTC_INT8>(h, d_frame, d_dm_out, d_s_meas, head, st, fh);
+        case RTC_F32: return launch_dt<RTC_F32>(h, d_frame, d_dm_out, d_s_meas, head, st, fh, d_s2);
+        case RTC_BF16: return launch_dt<RTC_BF16>(h, d_frame, d_dm_out, d_s_meas, head, st, fh, d_s2);
+        case RTC_F16: return launch_dt<RTC_F16>(h, d_frame, d_dm_out, d_s_meas, head, st, fh, d_s2);
+        case RTC_FP8_E4M3: return launch_dt<RTC_FP8_E4M3>(h, d_frame, d_dm_out, d_s_meas, head, st, fh, d_s2);
+        case RTC_INT8: return launch_dt<RTC_INT8>(h, d_frame, d_dm_out, d_s_meas, head, st, fh, d_s2);
         default: return cudaErrorInvalidValue;
     }
 }

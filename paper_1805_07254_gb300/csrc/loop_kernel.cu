@@ -411,7 +411,7 @@ cudaError_t launch_dt(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st) {
     const Launch Lc = plan_launch(h, pred ? rtc_pred::kSmemBytes : 0);
     if (!Lc.ok || Lc.G > h->dev_sms) return cudaErrorInvalidValue;
     LoopArgs a{};
-    a.px = pixel_args(h, nullptr, nullptr);
+    a.px = pixel_args(h, nullptr, nullptr, nullptr);
     a.mv = make_args(h, nullptr, nullptr, Lc);
     if (ll.l2_stream) a.mv.l2_policy = kL2Stream;
     a.frames = ll.d_frames;

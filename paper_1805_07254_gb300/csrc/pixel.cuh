@@ -1,7 +1,7 @@
 // Device code of the pixel stage (Sec. 2.1, Fig. 3 (a)-(b)), shared by the
 // stand-alone centroid kernel and the fused frame kernel.
 //
-// One warp takes one valid subaperture of one WFS.  The stage is latency-bound
+// A warp or half-warp takes one valid subaperture of one WFS.  The stage is latency-bound
 // (a 740x740 frame plus its calibration data is ~4 MB), so every lane issues all
 // of its loads -- raw pixels from the frame, dark and gain values from the
 // subap-major calibration arrays -- before any arithmetic.  Each lane then
@@ -55,6 +55,7 @@ struct PixelArgs {
     int thr_mode;
     float thr;
     float* s;                // [n_wfs][2][n_valid]
+    float* s2;               // a second copy of the slopes (the caller's buffer), or null
 };
 
 // How raw pixels are read: through the read-only path (a frame that does not change
@@ -82,20 +83,23 @@ struct NoHook {
 // frame and s_out: this frame's pixels and slope vector (PixelArgs' own fields are
 // not used, so that a persistent kernel can switch buffers per frame cheaply).
 // loaded(): called by every lane after each pass has issued its loads (the
-// passes are the same for every lane, valid or not).  Returns (x, y) slopes on the
-// group's first lane (zeros elsewhere).
+// passes are the same for every lane, valid or not).  ready(): called before each
+// pass's pixel loads, after its calibration loads (a kernel that may start before its
+// predecessor has finished waits there: the maps do not change while kernels run, the
+// frame may).  Returns (x, y) slopes on the group's first lane (zeros elsewhere).
 //
-// subap_slopes_at takes the subaperture's grid position (subap_pos) from the
-// caller, who may have loaded it early; subap_slopes loads it itself.
+// The subaperture's grid position (subap_pos) comes from the caller, who may have
+// loaded it early.
 __device__ __forceinline__ int2 subap_pos(const PixelArgs& p, int gi, bool valid) {
     const int w = valid ? gi / p.n_valid : 0;
     return valid ? p.rc[gi - w * p.n_valid] : make_int2(0, 0);
 }
 
-template <int NPX, int LD, int L, typename Hook = NoHook>
+template <int NPX, int LD, int L, typename Hook = NoHook, typename Ready = NoHook>
 __device__ __forceinline__ float2 subap_slopes_at(const PixelArgs& p, const uint16_t* __restrict__ frame,
                                                 float* __restrict__ s_out, int gi, bool valid, int lane,
-                                                int2 pos, const Hook& loaded = Hook()) {
+                                                int2 pos, const Hook& loaded = Hook(),
+                                                Ready ready = Ready()) {
     constexpr int kJ = NPX > 0 ? (NPX * NPX + L - 1) / L : kPixPerLane;
     const int npx = NPX > 0 ? NPX : p.npx;
     const int l = lane & (L - 1);
@@ -122,6 +126,7 @@ __device__ __forceinline__ float2 subap_slopes_at(const PixelArgs& p, const uint
                 gv[j] = __ldg(gk + q);
             }
         }
+        ready();
 #pragma unroll
         for (int j = 0; j < kJ; ++j) {
             const int q = q0 + l + L * j;
@@ -163,15 +168,13 @@ __device__ __forceinline__ float2 subap_slopes_at(const PixelArgs& p, const uint
         float* s_w = s_out + static_cast<size_t>(w) * 2 * p.n_valid;
         s_w[i] = res.x;
         s_w[p.n_valid + i] = res.y;
+        if (p.s2) {
+            float* s2_w = p.s2 + static_cast<size_t>(w) * 2 * p.n_valid;
+            s2_w[i] = res.x;
+            s2_w[p.n_valid + i] = res.y;
+        }
     }
     return res;
-}
-
-template <int NPX, int LD, int L, typename Hook = NoHook>
-__device__ __forceinline__ float2 subap_slopes(const PixelArgs& p, const uint16_t* __restrict__ frame,
-                                             float* __restrict__ s_out, int gi, bool valid, int lane,
-                                             const Hook& loaded = Hook()) {
-    return subap_slopes_at<NPX, LD, L>(p, frame, s_out, gi, valid, lane, subap_pos(p, gi, valid), loaded);
 }
 
 // ---- frame ingest from host memory ---------------------------------------------
@@ -239,4 +242,4 @@ __device__ __forceinline__ void ingest_block(const uint16_t* frame, uint16_t* st
 }  // namespace rtc_pixel
 
 // Pixel-stage arguments of a handle for one frame (defined in calib_cog.cu).
-rtc_pixel::PixelArgs pixel_args(const rtc_handle* h, const uint16_t* d_frame, float* d_s);
+rtc_pixel::PixelArgs pixel_args(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2);

@@ -2,6 +2,7 @@
 // map, calibration maps and control matrix, and the per-frame step.
 // Declarations and their contracts are in include/rtc.h.
 
+#include <cuda.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -265,25 +266,66 @@ int check_ready(rtc_handle* h) {
     return RTC_OK;
 }
 
+// Whether [a, a + an) and [b, b + bn) share a byte.
+bool overlap(const void* a, size_t an, const void* b, size_t bn) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + bn && y < x + an;
+}
+
+// Whether the kernels can write the slopes straight into `out`: float-aligned device
+// memory of the handle's device that holds all of them and shares no byte with what
+// else the call reads or writes.  Anything else goes through a copy, which checks it.
+bool slopes_direct(const rtc_handle* h, const float* out, const uint16_t* d_frame, const float* d_dm_out) {
+    typedef CUresult (*get_fn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+    static const get_fn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<get_fn>(f);
+    }();
+    const uintptr_t p = reinterpret_cast<uintptr_t>(out);
+    const size_t bytes = h->nslopes * sizeof(float);
+    if (!get || p % sizeof(float) != 0) return false;
+    CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned type = 0;
+    int dev = -1;
+    unsigned long long start = 0;
+    size_t size = 0;
+    void* to[4] = {&type, &dev, &start, &size};
+    if (get(4, what, to, p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || dev != h->cfg.device || p < start ||
+        p + bytes > start + size)
+        return false;
+    const size_t fbytes = static_cast<size_t>(h->cfg.n_wfs) * h->side * h->side * sizeof(uint16_t);
+    return !overlap(out, bytes, d_frame, fbytes) && !overlap(out, bytes, d_dm_out, h->cfg.nact * sizeof(float)) &&
+           !overlap(out, bytes, h->d_s, bytes);
+}
+
 // s_used (optional) receives the device buffer that holds this frame's measured slopes.
 int enqueue_step(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float* d_slopes_out,
                  cudaStream_t st, const float** s_used = nullptr, FrameHost* fh = nullptr) {
     if (s_used) *s_used = h->d_s;
+    float* direct = d_slopes_out && h->kpad > 0 && slopes_direct(h, d_slopes_out, d_frame, d_dm_out) ? d_slopes_out : nullptr;
     if (h->pred_on && h->kpad > 0) {
         // measured slopes into the next row of the history ring, the prediction from
         // the 4 newest rows, the reconstruction from the prediction: one launch
         const int head = (h->ring_head + 1) & 3;
         float* s_meas = h->d_ring + static_cast<size_t>(head) * h->kpad;
-        RTC_CUDA(h, launch_frame(h, d_frame, d_dm_out, s_meas, head, st, fh));
+        RTC_CUDA(h, launch_frame(h, d_frame, d_dm_out, s_meas, head, st, fh, direct));
         h->ring_head = head;
         if (s_used) *s_used = s_meas;
-        if (d_slopes_out)
+        if (d_slopes_out && !direct)
             RTC_CUDA(h, cudaMemcpyAsync(d_slopes_out, s_meas, h->nslopes * sizeof(float),
                                         cudaMemcpyDeviceToDevice, st));
         return RTC_OK;
     }
-    RTC_CUDA(h, launch_frame(h, d_frame, d_dm_out, nullptr, 0, st, fh));
-    if (d_slopes_out)
+    RTC_CUDA(h, launch_frame(h, d_frame, d_dm_out, nullptr, 0, st, fh, direct));
+    if (d_slopes_out && !direct)
         RTC_CUDA(h, cudaMemcpyAsync(d_slopes_out, h->d_s, h->nslopes * sizeof(float),
                                     cudaMemcpyDeviceToDevice, st));
     return RTC_OK;
@@ -847,8 +889,9 @@ int rtc_centroid_async(rtc_handle* h, const uint16_t* d_frame, float* d_slopes_o
     if (reinterpret_cast<uintptr_t>(d_frame) & 15) return fail(h, RTC_EINVAL, "d_frame must be 16-byte aligned");
     DeviceScope ds(h->cfg.device);
     cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : h->stream;
-    RTC_CUDA(h, launch_calib_cog(h, d_frame, h->d_s, st));
-    if (d_slopes_out)
+    float* direct = d_slopes_out && h->kpad > 0 && slopes_direct(h, d_slopes_out, d_frame, nullptr) ? d_slopes_out : nullptr;
+    RTC_CUDA(h, launch_calib_cog(h, d_frame, h->d_s, direct, st));
+    if (d_slopes_out && !direct)
         RTC_CUDA(h, cudaMemcpyAsync(d_slopes_out, h->d_s, h->nslopes * sizeof(float),
                                     cudaMemcpyDeviceToDevice, st));
     return RTC_OK;

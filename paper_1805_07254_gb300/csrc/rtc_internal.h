@@ -153,8 +153,8 @@ struct rtc_handle {
 };
 
 // Pixel calibration + centre of gravity + slope packing for every valid
-// subaperture of every WFS frame.  Writes s[0 .. nslopes).
-cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s,
+// subaperture of every WFS frame.  Writes s[0 .. nslopes) and, unless null, s2.
+cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2,
                              cudaStream_t st);
 
 // Slice-by-slice reconstruction (TMA bulk copies) with the fixed-order sum of the
@@ -177,9 +177,10 @@ cudaError_t launch_loop(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st);
 // h->d_s).  Otherwise the predictor path: measured slopes into d_s_meas = ring row
 // `head` of h->d_ring, predicted slopes into h->d_spred, reconstruction from those.
 // fh (optional): the frame and d_dm_out are device views of mapped host memory, and
-// the launch writes fh->done when its commands are out.
+// the launch writes fh->done when its commands are out.  d_s2 (optional): a second copy
+// of the measured slopes, written by the kernel.
 cudaError_t launch_frame(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float* d_s_meas,
-                         int head, cudaStream_t st, FrameHost* fh = nullptr);
+                         int head, cudaStream_t st, FrameHost* fh = nullptr, float* d_s2 = nullptr);
 cudaError_t launch_mvm_integrate(rtc_handle* h, const float* d_s, float* d_dm_out,
                                  cudaStream_t st);
 
