@@ -19,16 +19,27 @@ namespace {
 
 constexpr int kPerBlock = kCalibThreads / 16;
 
-template <int NPX>
+// EARLY: let the successor start at once (the prediction kernel, whose set-up and matrix
+// prefetch overlap this one); else after the wait: in a run of pixel stages alone,
+// waiting blocks of many later frames would fill the SMs (5.5 us a frame against 3.0).
+template <int NPX, bool EARLY>
 __global__ void __launch_bounds__(kCalibThreads) calib_cog_kernel(rtc_pixel::PixelArgs p) {
+    if (EARLY) pdl_launch_dependents();
     const int gi = blockIdx.x * kPerBlock + (threadIdx.x >> 4);
     const bool valid = gi < p.n_valid * p.n_wfs;
     const int2 pos = rtc_pixel::subap_pos(p, gi, valid);
-    rtc_pixel::subap_slopes_at<NPX, rtc_pixel::kPixelReadOnly, 16>(
+    rtc_pixel::subap_slopes_at<NPX, rtc_pixel::kPixelL2, 16>(
         p, p.frame, p.s, gi, valid, threadIdx.x & 31, pos, rtc_pixel::NoHook(), []() {
             pdl_wait();
-            pdl_launch_dependents();
+            if (!EARLY) pdl_launch_dependents();
         });
+}
+
+template <int NPX>
+cudaError_t launch_t(const rtc_pixel::PixelArgs& p, dim3 grid, bool early, cudaStream_t st) {
+    const dim3 block(kCalibThreads);
+    return early ? launch_pdl(calib_cog_kernel<NPX, true>, grid, block, 0, st, p)
+                 : launch_pdl(calib_cog_kernel<NPX, false>, grid, block, 0, st, p);
 }
 
 }  // namespace
@@ -38,16 +49,16 @@ rtc_pixel::PixelArgs pixel_args(const rtc_handle* h, const uint16_t* d_frame, fl
                                 h->d_dark, h->d_gainmap, h->thr_mode, h->thr,     d_s,          d_s2};
 }
 
-cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2,
+cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2, bool early,
                              cudaStream_t st) {
     const int n = h->n_valid * h->cfg.n_wfs;
     if (n == 0) return cudaSuccess;
-    const dim3 grid((n + kPerBlock - 1) / kPerBlock), block(kCalibThreads);
+    const dim3 grid((n + kPerBlock - 1) / kPerBlock);
     const rtc_pixel::PixelArgs p = pixel_args(h, d_frame, d_s, d_s2);
     switch (h->cfg.npx) {
-        case 8: return launch_pdl(calib_cog_kernel<8>, grid, block, 0, st, p);
-        case 10: return launch_pdl(calib_cog_kernel<10>, grid, block, 0, st, p);
-        case 16: return launch_pdl(calib_cog_kernel<16>, grid, block, 0, st, p);
-        default: return launch_pdl(calib_cog_kernel<0>, grid, block, 0, st, p);
+        case 8: return launch_t<8>(p, grid, early, st);
+        case 10: return launch_t<10>(p, grid, early, st);
+        case 16: return launch_t<16>(p, grid, early, st);
+        default: return launch_t<0>(p, grid, early, st);
     }
 }

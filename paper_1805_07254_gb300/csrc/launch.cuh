@@ -2,8 +2,10 @@
 // while the stream's previous kernel still runs (if that kernel lets it, or drains).
 // Its blocks call pdl_wait() before they read or write anything another kernel may
 // touch: it returns once the previous kernel has completed and its writes are visible.
-// A kernel calls pdl_launch_dependents() only after its own pdl_wait(), so that
-// whatever precedes it in the stream is complete before its successor starts.
+// (Loads of such data go through L2 or the ordinary path, never the read-only one.)
+// Before the wait a block touches only what no kernel writes.  Where a kernel calls
+// pdl_launch_dependents() after its own wait instead of first, its successor may also
+// rely on everything before it in the stream (the update of the predictor's training).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -92,7 +92,7 @@ constexpr unsigned long long kPollSpreadNs = 1200;
 
 struct LoopArgs {
     rtc_pixel::PixelArgs px;           // frame and s are set per frame
-    Args mv;                           // s and dm_out are set per frame
+    Args mv;                           // s is set per frame
     const uint16_t* frames;            // mapped host ring [nslot][frame_elems]
     unsigned long long frame_elems;
     uint16_t* stage;                   // device [frame_elems]: this frame's pixels
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
             consumer_sync();
             if (tid == 0) grid_arrive(L.gridbar);
             rtc_pred::Regs pr;
-            rtc_pred::prefetch(L.pa, pl.scratch, tid, pl.g0, pl.g1, head, pr);   // overlaps the barrier's wait
+            rtc_pred::prefetch<true>(L.pa, pl.scratch, tid, pl.g0, pl.g1, head, pr);   // overlaps the barrier's wait
             if (tid == 0) grid_wait(L.gridbar, G * (kBarriers * k + 1), L.mv.status, &sh.abort_flag);
             consumer_sync();
             if (sh.abort_flag) {
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
                 local_index(L.mv, pl, gi, ix, iy);
                 return axis ? iy : ix;
             };
-            rtc_pred::predict(
+            rtc_pred::predict<true>(
                 L.pa, pl.scratch, tid, pl.g0, pl.g1, head, pr,
                 [&](int gi, int axis) { return pl.loc[slot_of(gi, axis)]; },
                 [&](int gi, int axis, float v) { pl.loc[slot_of(gi, axis)] = v; });
@@ -408,11 +408,11 @@ namespace {
 template <int DT>
 cudaError_t launch_dt(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st) {
     const bool pred = h->pred_on;
-    const Launch Lc = plan_launch(h, pred ? rtc_pred::kSmemBytes : 0);
+    const Launch Lc = plan_launch(h, pred ? rtc_pred::kSmemBytes : 0, true);
     if (!Lc.ok || Lc.G > h->dev_sms) return cudaErrorInvalidValue;
     LoopArgs a{};
     a.px = pixel_args(h, nullptr, nullptr, nullptr);
-    a.mv = make_args(h, nullptr, nullptr, Lc);
+    a.mv = make_args(h, nullptr, Lc);
     if (ll.l2_stream) a.mv.l2_policy = kL2Stream;
     a.frames = ll.d_frames;
     a.frame_elems = ll.frame_elems;

@@ -159,7 +159,7 @@ __device__ __forceinline__ void fill_rows(Smem& sm, const float* __restrict__ X,
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
         const int q = threadIdx.x + j * kThreads;
-        v[j] = q < ns * NF ? X[static_cast<size_t>(s0) * NF + q] : 0.f;
+        v[j] = q < ns * NF ? __ldcg(X + static_cast<size_t>(s0) * NF + q) : 0.f;
     }
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(MlpDev w, const 
     train_body(sm, w, B, parts, [&](int s0, int ns) {
         fill_rows(sm, X, s0, ns);
         for (int i = threadIdx.x; i < TM * NO; i += kThreads)
-            sm.tgt[i / NO][i % NO] = i / NO < ns ? T[static_cast<size_t>(s0) * NO + i] : 0.f;
+            sm.tgt[i / NO][i % NO] = i / NO < ns ? __ldcg(T + static_cast<size_t>(s0) * NO + i) : 0.f;
     });
 }
 

@@ -1,10 +1,24 @@
-// Stand-alone reconstruction kernel (d = M s and the leaky integrator, Fig. 3
-// (c)-(d)) on a full slope vector; the device code is in stream_mvm.cuh.  Used by
-// rtc_reconstruct_async; rtc_process_frame runs the fused frame kernel, which gives
-// the same results bit for bit (same slices, same partials, same sum).  One
-// cooperative launch: each block gathers its slices' slopes, streams their matrix
-// bytes into partial vectors, and after a grid barrier reduces its share of rows.
+// The sum of the partial DM vectors, and the stand-alone reconstruction (d = M s and the
+// leaky integrator, Fig. 3 (c)-(d)) on a full slope vector.
+//
+// A per-frame call is two kernels: one writes a partial DM vector per matrix slice
+// (frame_kernel.cu, or mvm_stream_kernel here for rtc_reconstruct_async), the other
+// sums them (mvm_reduce_kernel).  The end of the first kernel is the barrier between
+// them, so no block ever waits for another one: nothing has to be co-resident, and the
+// launches need not be cooperative ones, which start only on an idle device.  Both are
+// launched with programmatic dependent launch and let their successor start at once:
+//   - the sum's blocks are small enough to sit on the SMs beside the streaming blocks
+//     and wait there, in hardware, for the partials;
+//   - the next frame's streaming blocks start as soon as this frame's leave their SM:
+//     their set-up and the fill of the ring (30 MB of the next matrix stream) run during
+//     the slowest blocks, the sum, and the hand-over, and they wait only before they
+//     read pixels.
+// Everything a kernel reads before its wait is written by no kernel (matrix, slice
+// table, maps, row scales).  frame_kernel.cu has the figures of this and of one
+// cooperative kernel with a grid barrier, whose launch waited for an idle device.
 
+#include "launch.cuh"
+#include "pred_tile.cuh"
 #include "stream_mvm.cuh"
 
 namespace {
@@ -12,11 +26,11 @@ namespace {
 using namespace rtc_mvm;
 
 template <int DT>
-__global__ void __launch_bounds__(kThreads, 1)
-mvm_stream_kernel(Args g, unsigned long long* gridbar, unsigned long long target) {
+__global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
     if (tid == 0) init_shared(sh);
     __syncthreads();
     const Plan pl = make_plan(g, smem);
@@ -26,16 +40,75 @@ mvm_stream_kernel(Args g, unsigned long long* gridbar, unsigned long long target
     }
     clear_local(g, pl, tid);
     consumer_sync();
-    gather_local(g, pl, tid, g.s, false);
-    prefetch_rows<DT>(g, pl, tid);
+    pdl_wait();
+    gather_local(g, pl, tid, g.s, true);
     consumer_sync();
     consume<DT>(g, pl, sh, tid, 0);
-    rows_landed();
-    // every block's partial vectors before any block sums them
-    consumer_sync();
-    if (tid == 0) grid_barrier(gridbar, target, g.status, &sh.abort_flag);
-    consumer_sync();
-    if (!sh.abort_flag) reduce_rows<DT>(g, pl, tid, g.dm_out);
+}
+
+// 32 rows a block, one per lane; the order of reduce_rows (stream_mvm.cuh).  A step that
+// a bounded wait cut short (status) leaves the integrator as it was.  HOST: the last
+// block to finish writes the caller's completion record.
+struct SumArgs {
+    const float* partial;    // [S][nact]
+    const float* scale;      // [nact] row scales, or null
+    float* a;
+    float* dm_out;           // [nact] or null
+    int* status;
+    int S, nact;
+    float gain, leak;
+};
+
+template <bool HOST>
+__global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, FrameHost fh) {
+    __shared__ float red[kConsumerWarps * 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int row = blockIdx.x * 32 + lane;
+    pdl_launch_dependents();
+    const bool mine = warp == 0 && row < r.nact;
+    const float sc = mine && r.scale ? __ldg(r.scale + row) : 1.f;
+    pdl_wait();
+    float a_prev = 0.f;
+    int status = 0;
+    if (mine) {
+        a_prev = __ldcg(r.a + row);
+        status = *reinterpret_cast<volatile int*>(r.status);
+    }
+    // the warp's slices w, w + 14, ...: 11 in flight (152 slices are one round)
+    constexpr int kFlight = 11;
+    float v = 0.f;
+    if (row < r.nact) {
+        for (int s0 = warp; s0 < r.S; s0 += kFlight * kConsumerWarps) {
+            float p[kFlight];
+#pragma unroll
+            for (int j = 0; j < kFlight; ++j) {
+                const int s = s0 + j * kConsumerWarps;
+                p[j] = s < r.S ? __ldcg(r.partial + static_cast<size_t>(s) * r.nact + row) : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < kFlight; ++j)
+                if (s0 + j * kConsumerWarps < r.S) v += p[j];
+        }
+    }
+    red[warp * 32 + lane] = v;
+    __syncthreads();
+    if (mine && status == 0) {
+        float t[kConsumerWarps];
+#pragma unroll
+        for (int w = 0; w < kConsumerWarps; ++w) t[w] = red[w * 32 + lane];
+#pragma unroll
+        for (int width = 1; width < kConsumerWarps; width <<= 1)
+#pragma unroll
+            for (int i = 0; i + width < kConsumerWarps; i += 2 * width) t[i] += t[i + width];
+        const float d = r.scale ? t[0] * sc : t[0];
+        const float an = fmaf(r.leak, a_prev, r.gain * d);
+        r.a[row] = an;
+        if (r.dm_out) r.dm_out[row] = an;
+    }
+    if (HOST) {
+        __syncthreads();
+        if (tid == 0) finish_host(fh, r.status);
+    }
 }
 
 // With no slopes, d = 0: only the leak acts.
@@ -51,16 +124,11 @@ __global__ void decay_kernel(int nact, float* __restrict__ a, float* __restrict_
 
 template <int DT>
 cudaError_t launch_stream(rtc_handle* h, const float* d_s, float* d_dm_out, cudaStream_t st) {
-    const Launch L = plan_launch(h);
+    const Launch& L = frame_plan(h, rtc_pred::kSmemBytes, false);
     if (!L.ok) return cudaErrorInvalidValue;
-    Args g = make_args(h, d_s, d_dm_out, L);
-    unsigned long long* bar = h->d_gridbar;
-    unsigned long long target = h->grid_epoch + static_cast<unsigned long long>(L.G);
-    void* args[] = {&g, &bar, &target};
-    const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(mvm_stream_kernel<DT>),
-                                                      dim3(L.G), dim3(kThreads), args, L.smem, st);
-    if (e == cudaSuccess) h->grid_epoch = target;
-    return e;
+    const Args g = make_args(h, d_s, L);
+    const cudaError_t e = launch_pdl(mvm_stream_kernel<DT>, dim3(L.G), dim3(kThreads), L.smem, st, g);
+    return e == cudaSuccess ? launch_sum(h, d_dm_out, st) : e;
 }
 
 template <int DT>
@@ -70,6 +138,18 @@ cudaError_t configure_one() {
 }
 
 }  // namespace
+
+cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {
+    const bool scaled = h->store == RTC_FP8_E4M3 || h->store == RTC_INT8;
+    const SumArgs r{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a, d_dm_out, h->d_status, h->sl_S,
+                    h->cfg.nact,  h->gain,                       h->leak};
+    const dim3 grid((h->cfg.nact + 31) / 32), block(kConsumers);
+    if (!fh) return launch_pdl(mvm_reduce_kernel<false>, grid, block, 0, st, r, FrameHost{});
+    fh->target = h->pf_arrivals + grid.x;
+    const cudaError_t e = launch_pdl(mvm_reduce_kernel<true>, grid, block, 0, st, r, *fh);
+    if (e == cudaSuccess) h->pf_arrivals = fh->target;
+    return e;
+}
 
 cudaError_t mvm_stream_configure() {
     cudaError_t e = configure_one<RTC_F32>();

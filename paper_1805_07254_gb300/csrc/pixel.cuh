@@ -58,17 +58,15 @@ struct PixelArgs {
     float* s2;               // a second copy of the slopes (the caller's buffer), or null
 };
 
-// How raw pixels are read: through the read-only path (a frame that does not change
-// while the kernel runs), fetched fresh every time (a frame buffer that a host
-// producer rewrites while a persistent kernel keeps running), or through L2 (a
-// device buffer that other blocks of the same kernel rewrite frame after frame).
-enum PixelLoad { kPixelReadOnly = 0, kPixelVolatile = 1, kPixelL2 = 2 };
+// How raw pixels are read: fetched fresh every time (a frame buffer that a host
+// producer rewrites while a persistent kernel keeps running), or through L2 (a device
+// buffer that other blocks of the same kernel, or a kernel that this one overlaps with
+// until its wait, may write: not through the read-only path).
+enum PixelLoad { kPixelVolatile = 1, kPixelL2 = 2 };
 
 template <int LD>
 __device__ __forceinline__ uint16_t load_pixel(const uint16_t* ptr) {
-    if (LD == kPixelVolatile) return __ldcv(ptr);
-    if (LD == kPixelL2) return __ldcg(ptr);
-    return __ldg(ptr);
+    return LD == kPixelVolatile ? __ldcv(ptr) : __ldcg(ptr);
 }
 
 struct NoHook {

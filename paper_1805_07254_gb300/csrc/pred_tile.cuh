@@ -21,12 +21,6 @@
 
 #include "stream_mvm.cuh"
 
-#ifndef RTC_PRED_STAMP
-#define RTC_PRED_STAMP(i) \
-    do {                  \
-    } while (0)
-#endif
-
 namespace rtc_pred {
 
 using rtc_mvm::consumer_sync;
@@ -114,7 +108,8 @@ __device__ __forceinline__ float gelu(float z) {
     return __fmaf_rn(-0.5f, __fmul_rn(a, gelu_erfc(a)), relu_nan(z));
 }
 
-// Two GELUs with packed FP32 arithmetic: the same bits as gelu() of each.
+// Two GELUs with packed FP32 arithmetic: the same bits as gelu() of each.  (For
+// throughput; its packed constants take 20 registers, which the fused kernels lack.)
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float lo, float hi) {
     f32x2 v;
@@ -183,7 +178,10 @@ __device__ __forceinline__ int pair_nbr(const PredArgs& pa, int t0, int i1, int 
 // frames) in registers, and the output layer's weights in the scratch sm
 // (asynchronous copies, complete once predict's first barrier has passed).
 // [i0, i1): the block's subapertures.  Call it after the block's grid-barrier
-// arrival (a release would wait for these loads) and before its wait.
+// arrival (a release would wait for these loads) and before its wait.  OLDER = false
+// leaves the older frames' features to predict: a kernel that may start before the
+// kernels that wrote those rows are known to be complete.
+template <bool OLDER>
 __device__ __forceinline__ void prefetch(const PredArgs& pa, unsigned char* sm, int tid, int i0, int i1,
                                          int head, Regs& r) {
     float* w3s = reinterpret_cast<float*>(sm + SM_W3);
@@ -212,6 +210,7 @@ __device__ __forceinline__ void prefetch(const PredArgs& pa, unsigned char* sm, 
     }
 #pragma unroll
     for (int q = 0; q < kPairRounds; ++q) r.jn[q] = pair_nbr(pa, i0, i1, tid + q * kConsumers);
+    if constexpr (OLDER)
 #pragma unroll
     for (int q = 0; q < kPairRounds; ++q)
 #pragma unroll
@@ -229,7 +228,7 @@ __device__ __forceinline__ void prefetch(const PredArgs& pa, unsigned char* sm, 
 // own copy of the measured slope s_k of subaperture i (the value in ring row head);
 // each prediction goes to pa.s_pred and to sink(i, axis, value), after the same
 // thread's src read of that slope.  Ends with a consumer barrier.
-template <typename Src, typename Sink>
+template <bool OLDER, typename Src, typename Sink>
 __device__ __forceinline__ void predict(const PredArgs& pa, unsigned char* sm, int tid, int i0, int i1,
                                         int head, const Regs& r, const Src& src, const Sink& sink) {
     const int warp = tid >> 5, lane = tid & 31;
@@ -244,22 +243,22 @@ __device__ __forceinline__ void predict(const PredArgs& pa, unsigned char* sm, i
     for (int lag = 0; lag < 4; ++lag)
         rows[lag] = pa.ring + static_cast<size_t>((head - lag) & 3) * pa.kpad;
 
-    RTC_PRED_STAMP(0);
     for (int t0 = i0; t0 < i1; t0 += TS) {
         int jn[kPairRounds];
 #pragma unroll
         for (int q = 0; q < kPairRounds; ++q)
             jn[q] = t0 == i0 ? r.jn[q] : pair_nbr(pa, t0, i1, tid + q * kConsumers);
         // gather: every load of the thread's pairs in flight before any store; the
-        // newest row was written by other blocks of this kernel, so it is read from
-        // L2 (the first tile's older rows came with prefetch)
+        // newest row was written by other blocks of this kernel (or by the kernel
+        // before it), so it is read from L2 (the first tile's older rows may have come
+        // with prefetch)
         float v[kPairRounds][8];
 #pragma unroll
         for (int q = 0; q < kPairRounds; ++q)
 #pragma unroll
             for (int la = 0; la < 8; ++la) {
                 const int j = jn[q];
-                if (la >= 2 && t0 == i0) v[q][la] = r.vo[q][la - 2];
+                if (OLDER && la >= 2 && t0 == i0) v[q][la] = r.vo[q][la - 2];
                 else v[q][la] = j >= 0 ? __ldcg(rows[la >> 1] + (la & 1) * pa.nv + j) : 0.f;
             }
 #pragma unroll
@@ -274,7 +273,6 @@ __device__ __forceinline__ void predict(const PredArgs& pa, unsigned char* sm, i
         }
         if (t0 == i0) rtc_mvm::rows_landed();     // the output layer's weights (prefetch)
         consumer_sync();
-        RTC_PRED_STAMP(1);
 
         // hidden layer 1: z1 = X W1^T + b1, h1 = GELU(z1) as BF16; the upper half of
         // the last k step is the zero padding of W1 and X (not stored: zero fragments)
@@ -296,12 +294,11 @@ __device__ __forceinline__ void predict(const PredArgs& pa, unsigned char* sm, i
 #pragma unroll
                 for (int h = 0; h < 4; h += 2) {
                     const int row = mt * 16 + g + (h >> 1) * 8, col = warp * 8 + 2 * t;
-                    const float2 v = gelu2(acc[mt][h] + r.b1v[0], acc[mt][h + 1] + r.b1v[1]);
-                    *reinterpret_cast<__nv_bfloat162*>(H1 + row * HP + col) = __floats2bfloat162_rn(v.x, v.y);
+                    *reinterpret_cast<__nv_bfloat162*>(H1 + row * HP + col) =
+                        __floats2bfloat162_rn(gelu(acc[mt][h] + r.b1v[0]), gelu(acc[mt][h + 1] + r.b1v[1]));
                 }
         }
         consumer_sync();
-        RTC_PRED_STAMP(2);
 
         // hidden layer 2: z2 = h1 W2^T + b2, h2 = GELU(z2) in FP32
         if (warp < kMmaWarps) {
@@ -321,34 +318,34 @@ __device__ __forceinline__ void predict(const PredArgs& pa, unsigned char* sm, i
                 for (int h = 0; h < 4; h += 2) {
                     const int row = mt * 16 + g + (h >> 1) * 8, col = warp * 8 + 2 * t;
                     *reinterpret_cast<float2*>(H2 + row * H2P + col) =
-                        gelu2(acc[mt][h] + r.b2v[0], acc[mt][h + 1] + r.b2v[1]);
+                        make_float2(gelu(acc[mt][h] + r.b2v[0]), gelu(acc[mt][h + 1] + r.b2v[1]));
                 }
         }
         consumer_sync();
-        RTC_PRED_STAMP(3);
 
-        // output layer on CUDA cores and the predicted next slopes: four lanes per
-        // output, lane t the columns 8 n + 2 t and 8 n + 2 t + 1 in order, then the
-        // four sums pairwise (the order of the sequence kernel, whose accumulator
-        // fragments hold those columns)
-        if (tid < TS * NO * 4) {
-            const int s = tid >> 3, o = (tid >> 2) & 1;
+        // output layer on CUDA cores and the predicted next slopes: the sum over the
+        // columns 8 n + 2 t and 8 n + 2 t + 1 for each t, then the four sums pairwise
+        // (the order of the sequence kernel, whose accumulator fragments hold those
+        // columns lane by lane)
+        if (tid < TS * NO) {
+            const int s = tid >> 1, o = tid & 1;
             const int i = t0 + s;
-            const float2* h = reinterpret_cast<const float2*>(H2 + s * H2P) + t;
-            const float2* c = reinterpret_cast<const float2*>(W3 + o * NH) + t;
-            float y = 0.f;
+            if (i < i1) {
+                float y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+                for (int n = 0; n < NH / 8; ++n)
 #pragma unroll
-            for (int n = 0; n < NH / 8; ++n) y = fmaf(h[4 * n].y, c[4 * n].y, fmaf(h[4 * n].x, c[4 * n].x, y));
-            y += __shfl_xor_sync(0xffffffffu, y, 1);
-            y += __shfl_xor_sync(0xffffffffu, y, 2);
-            if (t == 0 && i < i1) {
-                const float sp = __fmaf_rn(pa.sigma, y + b3[o], src(i, o));
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 h = *reinterpret_cast<const float2*>(H2 + s * H2P + 8 * n + 2 * q);
+                        const float2 c = *reinterpret_cast<const float2*>(W3 + o * NH + 8 * n + 2 * q);
+                        y[q] = fmaf(h.y, c.y, fmaf(h.x, c.x, y[q]));
+                    }
+                const float sp = __fmaf_rn(pa.sigma, ((y[0] + y[1]) + (y[2] + y[3])) + b3[o], src(i, o));
                 pa.s_pred[o * pa.nv + i] = sp;
                 sink(i, o, sp);
             }
         }
         consumer_sync();
-        RTC_PRED_STAMP(4);
     }
     if (i0 >= i1) rtc_mvm::rows_landed();         // no tile: still no copy left in flight
 }

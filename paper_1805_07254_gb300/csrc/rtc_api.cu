@@ -82,6 +82,7 @@ void free_slices(rtc_handle* h) {
     h->sl_g0.clear();
     h->sl_loc.clear();
     h->sl_equal = false;
+    h->plan_sms = 0;
     h->m_bytes = 0;
 }
 
@@ -132,7 +133,8 @@ void cut_slices(rtc_handle* h, const std::vector<int>& g0, int esz, std::vector<
     }
     h->sl_loc[S] = loc;
     h->m_bytes = off;
-    h->ingest_G = -1;                                   // the frame ingest follows the slices
+    h->ingest_G = -1;                                   // the frame ingest and the
+    h->plan_sms = 0;                                    // launch plans follow the slices
     // 1-byte stores take the plane layout when one lane per row holds (two ring
     // stages of kConsumers rows leave a generous margin of shared memory): their
     // rows then load as 16-byte units (measured: FP8 frame 21.0 against 22.5 us on
@@ -890,7 +892,7 @@ int rtc_centroid_async(rtc_handle* h, const uint16_t* d_frame, float* d_slopes_o
     DeviceScope ds(h->cfg.device);
     cudaStream_t st = stream ? static_cast<cudaStream_t>(stream) : h->stream;
     float* direct = d_slopes_out && h->kpad > 0 && slopes_direct(h, d_slopes_out, d_frame, nullptr) ? d_slopes_out : nullptr;
-    RTC_CUDA(h, launch_calib_cog(h, d_frame, h->d_s, direct, st));
+    RTC_CUDA(h, launch_calib_cog(h, d_frame, h->d_s, direct, false, st));
     if (d_slopes_out && !direct)
         RTC_CUDA(h, cudaMemcpyAsync(d_slopes_out, h->d_s, h->nslopes * sizeof(float),
                                     cudaMemcpyDeviceToDevice, st));

@@ -35,13 +35,13 @@ struct rtc_pf_done {
     int pad;
 };
 
-// What the frame kernel does for a caller waiting on the host (rtc_process_frame with
-// pinned buffers): the frame is read from mapped host memory, and the last block to
-// finish writes the completion record.
+// What the frame kernels do for a caller waiting on the host (rtc_process_frame with
+// pinned buffers): the frame is read from mapped host memory, and the last block of the
+// sum kernel writes the completion record.
 struct FrameHost {
     rtc_pf_done* done;           // device view of the mapped completion record
     unsigned long long* ctr;     // device count of finished blocks (only grows)
-    unsigned long long target;   // the count that completes this launch (set by launch_frame)
+    unsigned long long target;   // the count that completes this launch (set by launch_sum)
     unsigned long long seq;      // value of the record's seq for this call
     const unsigned* units;       // the blocks' copy units of the frame (build_ingest)
     const int4* blk;             // [G] first unit, end unit of each block
@@ -61,6 +61,13 @@ struct LoopLaunch {
     int nslot;
     int n_bands;                 // >= 1 bands of pixel rows per frame
     int l2_stream;               // stream the matrix with L2 evict_first whatever its size
+};
+
+// Grid, tiles, stages and dynamic shared memory of a streaming launch (stream_mvm.cuh).
+struct LaunchPlan {
+    int G, T, R, nst, stage_bytes, loc_floats, row_floats;
+    size_t smem, region;
+    bool ok;
 };
 
 struct rtc_handle {
@@ -97,6 +104,10 @@ struct rtc_handle {
     std::vector<int> sl_g0;         // [S + 1] first subaperture of each slice
     std::vector<int> sl_loc;        // [S + 1] float offset of each slice's slopes in a local vector
     bool sl_equal = false;          // sl_g0[s] == nt * s / S for every s
+    // the per-frame kernels' plans (without and with the predictor's scratch) for this
+    // slice table and plan_sms blocks; plan_sms is 0 when the table has changed
+    LaunchPlan plan[2]{};
+    int plan_sms = 0;
     bool sl_plane = false;          // slices stored in the plane layout (1- and 2-byte stores)
     long long* d_sl_off = nullptr;
     int* d_sl_rowbytes = nullptr;
@@ -153,8 +164,10 @@ struct rtc_handle {
 };
 
 // Pixel calibration + centre of gravity + slope packing for every valid
-// subaperture of every WFS frame.  Writes s[0 .. nslopes) and, unless null, s2.
-cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2,
+// subaperture of every WFS frame.  Writes s[0 .. nslopes) and, unless null, s2.  early:
+// the next kernel of the stream is one that reads nothing before its wait that a kernel
+// writes, and may start at once.
+cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float* d_s, float* d_s2, bool early,
                              cudaStream_t st);
 
 // Slice-by-slice reconstruction (TMA bulk copies) with the fixed-order sum of the
@@ -162,8 +175,11 @@ cudaError_t launch_calib_cog(const rtc_handle* h, const uint16_t* d_frame, float
 cudaError_t mvm_stream_configure();
 cudaError_t launch_decay(const rtc_handle* h, float* d_dm_out, cudaStream_t st);
 
-// Fused frame kernel (pixel stage + grid barrier + streaming MVM + integrator),
-// one cooperative launch per frame; the slopes land in h->d_s.
+// The sum of the partial DM vectors and the integrator (mvm_stream.cu), after the kernel
+// that wrote the partials.  fh (optional): its last block writes the completion record.
+cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh = nullptr);
+
+// Frame kernels (pixel stage + streaming MVM); the slopes land in h->d_s.
 cudaError_t frame_kernel_configure();
 
 // The per-block copy units of a frame for a G-block launch (loop_kernel.cu); rebuilt

@@ -12,10 +12,11 @@
 // kernel takes a run of whole slices and computes those subapertures' slopes
 // itself, so its share of the product starts as soon as its own pixels are done,
 // without waiting for any other block; it writes one partial vector per slice.
-// After one grid barrier every block sums the S partials of its share of the rows
-// in a fixed order (warp w sums the slices w, w+14, w+28, ... in turn for 32
-// consecutive rows with coalesced loads, then a fixed pairwise tree over the 14
-// warps), applies the FP8/INT8 row scale and the integrator.
+// Once every block is done the S partials of each row are summed in a fixed order (warp
+// w sums the slices w, w+14, w+28, ... in turn for 32 consecutive rows with coalesced
+// loads, then a fixed pairwise tree over the 14 warps), with the FP8/INT8 row scale
+// and the integrator: by the sum kernel that follows a per-frame kernel
+// (mvm_reduce_kernel), or after a grid barrier in the persistent loop.
 // The result does not depend on the number of blocks or on their timing.
 //
 // Movement.  A slice streams in tiles of R rows, bulk asynchronous copies
@@ -64,6 +65,11 @@ constexpr unsigned long long kWaitNs = 200ull * 1000 * 1000;
 constexpr int kMaxLocalFloats = 8192;              // slopes of a block's slices (32 KB)
 constexpr int kMaxRowFloats = 4096;                // rows a block reduces, at most
 constexpr size_t kDynSmemBudget = 227 * 1024 - 2048;  // dynamic shared memory per block
+// The per-frame kernels leave room on their SM for a block of the sum kernel
+// (mvm_reduce_kernel: 2 KB of shared memory, 448 threads of 32 registers, so at most 104
+// registers for theirs: the bound of 608 threads).
+constexpr size_t kFrameSmemBudget = 223 * 1024;
+constexpr int kFrameRegThreads = 608;
 constexpr int kMaxSlices = 256;
 constexpr int kSlicesPerWarp = (kMaxSlices + kConsumerWarps - 1) / kConsumerWarps;
 constexpr uint32_t kCopyBytes = 8192;              // largest single bulk copy of a tile
@@ -124,10 +130,6 @@ __device__ __forceinline__ unsigned long long matrix_policy(int mode) {
     else
         asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
     return p;
-}
-// Bulk prefetch of global bytes into L2 (no shared memory, no completion).
-__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
@@ -191,17 +193,6 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
         if (abort && *abort) return false;
         if (global_ns() - t0 > kWaitNs) return false;
     }
-}
-
-// Bounded wait for a shared-memory flag; false if it expired or the block aborted.
-__device__ __forceinline__ bool wait_flag(volatile int* flag, volatile int* abort) {
-    const unsigned long long t0 = global_ns();
-    while (!*flag) {
-        if (*abort) return false;
-        if (global_ns() - t0 > kWaitNs) return false;
-        __nanosleep(64);
-    }
-    return true;
 }
 
 // ---- widening dot products: acc += <one 4-byte word of a row, its slopes> -------
@@ -290,7 +281,6 @@ struct Args {
     const float* scale;      // [nact] row scales (FP8, INT8)
     float* partial;          // [S][nact] partial DM vectors
     float* a;                // [nact] integrator state
-    float* dm_out;           // [nact] or nullptr
     float gain, leak;
     int* status;             // device error word
 };
@@ -299,7 +289,6 @@ struct Shared {
     unsigned long long full_bar[kMaxStages];
     unsigned long long empty_bar[kMaxStages];
     volatile int abort_flag;
-    volatile int release;    // set once the block's slopes are known (see produce's hold)
 };
 
 // What one block does.
@@ -322,7 +311,6 @@ __device__ __forceinline__ void init_shared(Shared& sh) {
         mbar_init(smem_addr(&sh.empty_bar[i]), kConsumerWarps);
     }
     sh.abort_flag = 0;
-    sh.release = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
@@ -424,35 +412,13 @@ __device__ __forceinline__ int tile_rows(const Args& g, int rb) {
     return g.R * (m < 1 ? 1 : m > kMaxRowsPerThread ? kMaxRowsPerThread : m);
 }
 
-// Source and size of tile t of the block (counted from the start of its first
-// slice); false past its last tile.
-__device__ __forceinline__ bool tile_src(const Args& g, const Plan& pl, int t, const unsigned char*& src,
-                                         uint32_t& bytes) {
-    for (int s = pl.sb0; s < pl.sb1; ++s) {
-        const int rb = g.sl.rowbytes[s];
-        const int tr = tile_rows(g, rb);
-        const int nt = (g.nact + tr - 1) / tr;
-        if (t < nt) {
-            const int row0 = t * tr;
-            src = g.M + g.sl.off[s] + static_cast<size_t>(row0) * rb;
-            bytes = (static_cast<uint32_t>(min(tr, g.nact - row0)) * rb + 15u) & ~15u;
-            return true;
-        }
-        t -= nt;
-    }
-    return false;
-}
-
 // One producer thread: stream the block's slices tile by tile into the ring.
 // tl0: the running tile count at entry (barrier phases continue across calls, e.g.
 // frame after frame in a persistent kernel); returns the count at exit.  drain: wait
 // for the last copies to land before returning (a block must not exit with copies
-// in flight).  hold > 0: after the first `hold` tiles, wait until the consumers set
-// sh.release (the latency-critical pixel loads then do not queue behind the
-// stream).  hold_l2: tiles prefetched into L2 right before that wait (a long wait,
-// such as the predictor's, then leaves the HBM streaming).
-__device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh, int tl0 = 0,
-                                       bool drain = true, int hold = 0, int hold_l2 = 0) {
+// in flight).  The ring fills before the block's slopes are known and then waits for
+// its consumers.
+__device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh, int tl0 = 0, bool drain = true) {
     int tl = tl0;
     bool ok = true;
     const unsigned long long policy = matrix_policy(g.l2_policy);
@@ -461,17 +427,6 @@ __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh
         const int rb = g.sl.rowbytes[s];
         const int tr = tile_rows(g, rb);
         for (int row0 = 0; row0 < g.nact; row0 += tr, ++tl) {
-            if (hold > 0 && tl - tl0 == hold) {
-                for (int j = 0; j < hold_l2; ++j) {
-                    const unsigned char* psrc;
-                    uint32_t pbytes;
-                    if (tile_src(g, pl, hold + j, psrc, pbytes)) bulk_prefetch_l2(psrc, pbytes);
-                }
-                if (!wait_flag(&sh.release, &sh.abort_flag)) {
-                    ok = false;
-                    break;
-                }
-            }
             const int st = tl % g.nst;
             const int use = tl / g.nst;
             if (use > 0 && !wait_phase(smem_addr(&sh.empty_bar[st]), (use - 1) & 1, &sh.abort_flag)) {
@@ -825,16 +780,27 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* bar, unsigned l
     return grid_wait(bar, target, status, abort);
 }
 
-// Grid, tiles, stages and dynamic shared memory of a launch for one handle.
-struct Launch {
-    int G, T, R, nst, stage_bytes, loc_floats, row_floats;
-    size_t smem, region;
-    bool ok;
-};
+// One thread per block, after the block's commands are written: the last block to finish
+// writes the completion record of a caller waiting on the host (every block, aborted or
+// not, counts itself once).
+__device__ __forceinline__ void finish_host(const FrameHost& fh, const int* status) {
+    __threadfence_system();
+    const unsigned long long prev = atomicAdd(fh.ctr, 1ull);
+    if (prev + 1 == fh.target) {
+        __threadfence_system();
+        fh.done->status = *reinterpret_cast<const volatile int*>(status);
+        __threadfence_system();
+        asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"(&fh.done->seq), "l"(fh.seq) : "memory");
+    }
+}
 
-// min_region: shared-memory scratch a fused phase needs.  Uses the handle's slice
-// table, built when the matrix was loaded.
-inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0) {
+using Launch = LaunchPlan;
+
+// min_region: shared-memory scratch a fused phase needs.  loop: the persistent kernel,
+// which also sums its rows (integrator state, row scales and warp sums in shared
+// memory); the lanes per row are the same for both.  Uses the handle's slice table,
+// built when the matrix was loaded.
+inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop = false) {
     Launch L{};
     const int S = h->sl_S;
     L.G = S < h->num_sms ? S : h->num_sms;
@@ -850,9 +816,10 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0) {
     L.loc_floats = (max_loc + 3) / 4 * 4;
     L.row_floats = (h->cfg.nact + L.G - 1) / L.G;
     L.region = (min_region + 15) / 16 * 16;
-    const size_t extra = L.region + 4 * static_cast<size_t>(L.loc_floats) +
-                         8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
-    const size_t room = kDynSmemBudget > extra ? kDynSmemBudget - extra : 0;
+    size_t extra = L.region + 4 * static_cast<size_t>(L.loc_floats) +
+                   8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
+    size_t budget = kDynSmemBudget;
+    size_t room = budget > extra ? budget - extra : 0;
     // lanes per row: the fewest for which two stages of R = kConsumers / T rows fit
     // (splitting rows further to keep the slopes in registers measured slower for
     // every store type: more tiles and butterflies cost more than the slope reads
@@ -862,6 +829,12 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0) {
     L.T = 1;
     while (L.T < 16 && 2 * stage(L.T) > room) L.T *= 2;      // R stays a multiple of 4
     L.R = kConsumers / L.T;
+    if (!loop) {
+        extra = L.region + 4 * static_cast<size_t>(L.loc_floats);
+        // (a plan that would not get its two stages beside a sum block takes the whole SM)
+        budget = 2 * stage(L.T) + extra <= kFrameSmemBudget ? kFrameSmemBudget : kDynSmemBudget;
+        room = budget > extra ? budget - extra : 0;
+    }
     // stages of at least kMinTileBytes (whole multiples of R rows of the widest
     // slice), so that the per-tile handshakes stay a small part of the work
     const size_t st1 = stage(L.T);
@@ -872,11 +845,22 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0) {
     L.nst = static_cast<int>(fit < static_cast<size_t>(kMaxStages) ? fit : kMaxStages);
     L.smem = static_cast<size_t>(L.nst) * L.stage_bytes + extra;
     L.ok = L.nst >= 2 && L.loc_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
-           S <= kMaxSlices && L.smem <= kDynSmemBudget && (!h->sl_plane || L.T == 1);
+           S <= kMaxSlices && L.smem <= budget && (!h->sl_plane || L.T == 1);
     return L;
 }
 
-inline Args make_args(const rtc_handle* h, const float* d_s, float* d_dm_out, const Launch& L) {
+// The plan of a per-frame kernel, worked out once per slice table and block limit: the
+// walk over blocks and slices is 0.8 us of host time, a tenth of a small frame's call.
+inline const Launch& frame_plan(rtc_handle* h, size_t pred_region, bool pred) {
+    if (h->plan_sms != h->num_sms) {
+        h->plan[0] = plan_launch(h);
+        h->plan[1] = plan_launch(h, pred_region);
+        h->plan_sms = h->num_sms;
+    }
+    return h->plan[pred ? 1 : 0];
+}
+
+inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
     Args g{};
     g.M = static_cast<const unsigned char*>(h->d_M);
     g.sl = Slices{h->d_sl_off, h->d_sl_rowbytes, h->d_sl_g0, h->d_sl_loc, h->sl_S,
@@ -896,7 +880,6 @@ inline Args make_args(const rtc_handle* h, const float* d_s, float* d_dm_out, co
     g.scale = h->d_scale;
     g.partial = h->d_partial;
     g.a = h->d_a;
-    g.dm_out = d_dm_out;
     g.gain = h->gain;
     g.leak = h->leak;
     g.status = h->d_status;
