@@ -134,14 +134,16 @@ def _ptr(x):
     """Raw address of a numpy array or torch tensor (None -> NULL)."""
     if x is None:
         return None
+    try:                                   # tensors first: they are passed on every frame
+        if x.is_contiguous():
+            return x.data_ptr()
+        raise ValueError("tensors passed to librtc must be contiguous")
+    except AttributeError:
+        pass
     if isinstance(x, np.ndarray):
         if not x.flags["C_CONTIGUOUS"]:
             raise ValueError("arrays passed to librtc must be C-contiguous")
         return x.ctypes.data
-    if hasattr(x, "data_ptr"):
-        if not x.is_contiguous():
-            raise ValueError("tensors passed to librtc must be contiguous")
-        return x.data_ptr()
     if isinstance(x, int):
         return x
     raise TypeError(f"cannot pass {type(x)} to librtc")
@@ -157,9 +159,10 @@ def _stream_ptr(stream):
     """cudaStream_t for a torch stream, a raw handle, or None (the library default)."""
     if stream is None:
         return None
-    if hasattr(stream, "cuda_stream"):
+    try:
         return stream.cuda_stream or _CUDA_STREAM_LEGACY
-    return int(stream)
+    except AttributeError:
+        return int(stream)
 
 
 class Rtc:
@@ -286,13 +289,16 @@ class Rtc:
 
     def process_frame_async(self, d_frame, d_dm_out=None, d_slopes_out=None, stream=None):
         """Enqueue one step on device buffers (torch CUDA tensors) on ``stream``."""
-        self._check(self._lib.rtc_process_frame_async(self._h, _ptr(d_frame), _ptr(d_dm_out),
-                                                      _ptr(d_slopes_out), _stream_ptr(stream)))
+        rc = self._lib.rtc_process_frame_async(self._h, _ptr(d_frame), _ptr(d_dm_out), _ptr(d_slopes_out),
+                                               _stream_ptr(stream))
+        if rc:
+            self._check(rc)
 
     def centroid_async(self, d_frame, d_slopes_out=None, stream=None):
         """Enqueue the pixel stage (calibration + centroids) on device buffers."""
-        self._check(self._lib.rtc_centroid_async(self._h, _ptr(d_frame), _ptr(d_slopes_out),
-                                                 _stream_ptr(stream)))
+        rc = self._lib.rtc_centroid_async(self._h, _ptr(d_frame), _ptr(d_slopes_out), _stream_ptr(stream))
+        if rc:
+            self._check(rc)
 
     def reconstruct_async(self, d_slopes=None, d_dm_out=None, stream=None):
         """Enqueue MVM + integrator from ``d_slopes`` (None: the resident slope buffer)."""
