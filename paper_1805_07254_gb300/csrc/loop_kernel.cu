@@ -435,7 +435,7 @@ cudaError_t launch_dt(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st) {
     a.done = ll.d_done;
     a.s_buf = h->d_sbuf;
     a.gridbar = h->d_gridbar;
-    a.partial_stride = static_cast<size_t>(h->dev_sms) * h->cfg.nact;
+    a.partial_stride = static_cast<size_t>(h->dev_sms) * partial_pitch(h->cfg.nact);
     a.donectr = h->d_donectr;
     a.t_seen = h->d_tseen;
     a.n_frames = ll.n_frames;

@@ -50,12 +50,12 @@ __global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g)
 // a bounded wait cut short (status) leaves the integrator as it was.  HOST: the last
 // block to finish writes the caller's completion record.
 struct SumArgs {
-    const float* partial;    // [S][nact]
+    const float* partial;    // [S][pitch]
     const float* scale;      // [nact] row scales, or null
     float* a;
     float* dm_out;           // [nact] or null
     int* status;
-    int S, nact;
+    int S, nact, pitch;
     float gain, leak;
 };
 
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, Fr
 #pragma unroll
             for (int j = 0; j < kFlight; ++j) {
                 const int s = s0 + j * kConsumerWarps;
-                p[j] = s < r.S ? __ldcg(r.partial + static_cast<size_t>(s) * r.nact + row) : 0.f;
+                p[j] = s < r.S ? __ldcg(r.partial + static_cast<size_t>(s) * r.pitch + row) : 0.f;
             }
 #pragma unroll
             for (int j = 0; j < kFlight; ++j)
@@ -141,8 +141,8 @@ cudaError_t configure_one() {
 
 cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {
     const bool scaled = h->store == RTC_FP8_E4M3 || h->store == RTC_INT8;
-    const SumArgs r{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a, d_dm_out, h->d_status, h->sl_S,
-                    h->cfg.nact,  h->gain,                       h->leak};
+    const SumArgs r{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a,  d_dm_out, h->d_status, h->sl_S,
+                    h->cfg.nact,  partial_pitch(h->cfg.nact),    h->gain, h->leak};
     const dim3 grid((h->cfg.nact + 31) / 32), block(kConsumers);
     if (!fh) return launch_pdl(mvm_reduce_kernel<false>, grid, block, 0, st, r, FrameHost{});
     fh->target = h->pf_arrivals + grid.x;

@@ -104,14 +104,16 @@ std::vector<int> slice_bounds(const rtc_handle* h, int esz) {
 }
 
 // The slice table for slice bounds g0, in the handle's host vectors: each slice one
-// contiguous [nact][2 n_s] block (x slopes, then y slopes), rows padded to a
-// multiple of 4 bytes with an access unit (16, 8 or 4 bytes) that divides them an
-// odd number of times.  colmap: column c (WFS w, axis, subaperture i) -> (slice,
+// contiguous [nact][2 n_s] block (x slopes, then y slopes): FP32 rows padded until an
+// access unit (16, 8 or 4 bytes) divides them an odd number of times, 1- and 2-byte
+// stores unpadded in fragment order (rtc_mvm::slice_elem_offset).  colmap: column c (WFS w, axis, subaperture i) -> (slice,
 // column within the slice).
 void cut_slices(rtc_handle* h, const std::vector<int>& g0, int esz, std::vector<int2>& colmap) {
     const int S = static_cast<int>(g0.size()) - 1;
     const int nact = h->cfg.nact;
     h->sl_S = S;
+    h->sl_frag = esz < 4;
+    h->sl_esz = esz;
     h->sl_g0 = g0;
     h->sl_equal = true;
     for (int s = 0; s <= S; ++s)
@@ -123,26 +125,20 @@ void cut_slices(rtc_handle* h, const std::vector<int>& g0, int esz, std::vector<
     int loc = 0;
     for (int s = 0; s < S; ++s) {
         const int n = g0[s + 1] - g0[s];
-        int rb = (2 * n * esz + 3) / 4 * 4;
-        while (rtc_mvm::row_unit(rb) == 0) rb += 4;       // a bank-conflict-free access unit
+        int rb = 2 * n * esz;
+        if (!h->sl_frag)
+            while (rtc_mvm::row_unit(rb) == 0) rb += 4;   // a bank-conflict-free access unit
+        const long long rows = h->sl_frag ? (nact + 15) / 16 * 16ll : nact;
         h->sl_off[s] = off;
         h->sl_rowbytes[s] = rb;
-        off += (static_cast<long long>(nact) * rb + 15) / 16 * 16;
+        off += (rows * rb + 15) / 16 * 16;
         h->sl_loc[s] = loc;
-        loc += (rb / esz + 3) / 4 * 4;
+        loc += h->sl_frag ? (2 * n + 15) / 16 * 16 : (rb / esz + 3) / 4 * 4;
     }
     h->sl_loc[S] = loc;
     h->m_bytes = off;
     h->ingest_G = -1;                                   // the frame ingest and the
     h->plan_sms = 0;                                    // launch plans follow the slices
-    // 1-byte stores take the plane layout when one lane per row holds (two ring
-    // stages of kConsumers rows leave a generous margin of shared memory): their
-    // rows then load as 16-byte units (measured: FP8 frame 21.0 against 22.5 us on
-    // ELT; 2-byte stores, which keep up with the HBM anyway, gained nothing)
-    int max_rb = 0;
-    for (int s = 0; s < S; ++s) max_rb = std::max(max_rb, h->sl_rowbytes[s]);
-    h->sl_plane = esz == 1 && 2 * static_cast<long long>(rtc_mvm::kConsumers) * max_rb + (64 << 10) <=
-                                  static_cast<long long>(rtc_mvm::kDynSmemBudget);
     const int nv = h->n_valid, nt = nv * h->cfg.n_wfs;
     std::vector<int> slice_of(nt);
     for (int s = 0; s < S; ++s)
@@ -472,7 +468,7 @@ int rtc_create(const rtc_config* cfg, rtc_handle** out) {
     } else {
         const size_t frame_elems = static_cast<size_t>(c.n_wfs) * h->side * h->side;
         if (cudaMalloc(&h->d_a, c.nact * sizeof(float)) != cudaSuccess ||
-            cudaMalloc(&h->d_partial, 2 * static_cast<size_t>(h->dev_sms) * c.nact * sizeof(float)) != cudaSuccess ||
+            cudaMalloc(&h->d_partial, 2 * static_cast<size_t>(h->dev_sms) * partial_pitch(c.nact) * sizeof(float)) != cudaSuccess ||
             cudaMalloc(&h->d_frame, frame_elems * sizeof(uint16_t)) != cudaSuccess ||
             cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess ||
             cudaMalloc(&h->d_gridbar, sizeof(unsigned long long)) != cudaSuccess ||
@@ -646,7 +642,7 @@ int rtc_load_cmat(rtc_handle* h, const void* M, int32_t nact, int32_t nslopes, i
     if (e == cudaSuccess) e = cudaMemcpy(d_colmap, colmap.data(), nslopes * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = launch_layout(src, store, staging, nact, nslopes, d_colmap, h->d_sl_off, h->d_sl_rowbytes,
-                          h->sl_plane ? 1 : 0, h->d_scale, h->d_M, h->stream);
+                          h->d_scale, h->d_M, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     cudaFree(staging);
     cudaFree(d_colmap);
@@ -670,7 +666,6 @@ int rtc_set_readout(rtc_handle* h, int32_t n_bands, double band_interval_us) {
     const int nact = h->cfg.nact, ncol = h->nslopes;
     std::vector<int2> old_map, new_map;
     cut_slices(h, h->sl_g0, esz, old_map);                  // the present cut's column map
-    const int old_plane = h->sl_plane ? 1 : 0;
     const std::vector<int> g0 = slice_bounds(h, esz);
     void* old_M = h->d_M;
     long long* old_off = h->d_sl_off;
@@ -693,7 +688,7 @@ int rtc_set_readout(rtc_handle* h, int32_t n_bands, double band_interval_us) {
     if (e == cudaSuccess)
         e = cudaMemcpy(d_maps + ncol, new_map.data(), ncol * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_relayout(esz, old_plane, h->sl_plane ? 1 : 0, old_M, d_maps, old_off, old_rb, nact, ncol, d_maps + ncol,
+        e = launch_relayout(esz, old_M, d_maps, old_off, old_rb, nact, ncol, d_maps + ncol,
                             h->d_sl_off, h->d_sl_rowbytes, h->d_M, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (d_maps) cudaFree(d_maps);
@@ -864,7 +859,7 @@ int64_t rtc_handle_device_bytes(const rtc_handle* h) {
     int64_t b = h->m_bytes + 4 * nact;                                         // matrix + scales
     b += 2 * 4 * nw * h->n_valid * npp;                                        // dark + gain
     b += nw * static_cast<int64_t>(h->side) * h->side * 2;                     // frame staging
-    b += 4 * (kpad + nact) + 8 * static_cast<int64_t>(h->dev_sms) * nact + 4 * nact;  // s, a, partials
+    b += 4 * (kpad + nact) + 8 * static_cast<int64_t>(h->dev_sms) * partial_pitch(h->cfg.nact) + 4 * nact;  // s, a, partials
     if (h->pred) b += 4 * (5 * kpad) + 4 * 25 * h->n_valid + 3 * 4 * RTC_MLP_NPARAMS + 2 * (64 * 208 + 64 * 64);
     return b;
 }

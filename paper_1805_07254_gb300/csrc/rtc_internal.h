@@ -63,9 +63,12 @@ struct LoopLaunch {
     int l2_stream;               // stream the matrix with L2 evict_first whatever its size
 };
 
+// Floats from one slice's partial DM vector to the next: whole groups of 16 rows.
+inline int partial_pitch(int nact) { return (nact + 15) / 16 * 16; }
+
 // Grid, tiles, stages and dynamic shared memory of a streaming launch (stream_mvm.cuh).
 struct LaunchPlan {
-    int G, T, R, nst, stage_bytes, loc_floats, row_floats;
+    int G, T, R, nst, stage_bytes, loc_floats, row_floats, max_slices, bf_floats;
     size_t smem, region;
     bool ok;
 };
@@ -108,14 +111,15 @@ struct rtc_handle {
     // slice table and plan_sms blocks; plan_sms is 0 when the table has changed
     LaunchPlan plan[2]{};
     int plan_sms = 0;
-    bool sl_plane = false;          // slices stored in the plane layout (1- and 2-byte stores)
+    bool sl_frag = false;           // slices in fragment order (1- and 2-byte stores)
+    int sl_esz = 4;                 // bytes per stored entry
     long long* d_sl_off = nullptr;
     int* d_sl_rowbytes = nullptr;
     int* d_sl_g0 = nullptr;
     int* d_sl_loc = nullptr;
     float* d_s = nullptr;           // [kpad] slope vector, zero padded
     float* d_a = nullptr;           // [nact] integrator state
-    float* d_partial = nullptr;     // [2][dev_sms][nact] partial DM vectors, one per slice (scratch;
+    float* d_partial = nullptr;     // [2][dev_sms][pitch] partial DM vectors, one per slice (scratch;
                                     // the persistent loop alternates the halves frame by frame)
     uint16_t* d_frame = nullptr;    // [n_wfs][side][side] staging for host frames
     int* d_status = nullptr;        // device-side error word (RTC_ETIMEDOUT from bounded waits)
@@ -212,12 +216,12 @@ cudaError_t launch_mvm_raw(int store, const void* d_M, const float* d_scale, int
 // local column colmap[c].y.  From FP32, the FP8 / INT8 row scales are computed
 // into d_scale first.
 cudaError_t launch_layout(int src, int store, const void* d_src, int nact, int ncol,
-                          const int2* d_colmap, const long long* d_off, const int* d_rowbytes, int plane,
+                          const int2* d_colmap, const long long* d_off, const int* d_rowbytes,
                           float* d_scale, void* d_dst, cudaStream_t st);
 
 // Move a matrix between two slice layouts of the same store (esize bytes per
 // entry): column c from (old_colmap[c]) to (new_colmap[c]).
-cudaError_t launch_relayout(int esize, int old_plane, int new_plane, const void* d_old, const int2* d_old_colmap,
+cudaError_t launch_relayout(int esize, const void* d_old, const int2* d_old_colmap,
                             const long long* d_old_off, const int* d_old_rowbytes, int nact, int ncol,
                             const int2* d_new_colmap, const long long* d_new_off, const int* d_new_rowbytes,
                             void* d_new, cudaStream_t st);

@@ -20,20 +20,18 @@
 // The result does not depend on the number of blocks or on their timing.
 //
 // Movement.  A slice streams in tiles of R rows, bulk asynchronous copies
-// (`cp.async.bulk`) completing on a per-stage mbarrier, through a ring of up to 8
+// (`cp.async.bulk`) completing on a per-stage mbarrier, through a ring of up to 32
 // stages in shared memory that one producer thread fills and 14 consumer warps
-// drain.  T consecutive lanes take one row of a tile (T = 1 for ELT-sized slices,
-// more when rows are long, so that at least two stages fit) and read it in units of
-// 16, 8 or 4 bytes, the widest that divides the row an odd number of times (rows
-// are padded until one does), so that the rows a warp reads at once fall in
-// different banks; all lanes read the same units of the slice's slopes at the same
-// time (shared-memory broadcasts).
+// drain.
 //
-// Arithmetic.  Stored values are widened to FP32 just before the FMA (BF16 by a
-// shift, FP16 by the half2 -> float2 conversion, E4M3 by the hardware fp8x2 ->
-// f16x2 conversion, INT8 exactly through the mantissa of 2^23), as Sec. 2.3.4
-// widens its 16-bit matrix; the FP8 and INT8 row scales are applied once per row
-// after the sum over slices.
+// Arithmetic.  FP32 rows: T consecutive lanes take one row of a tile (T = 1 for
+// ELT-sized slices, more when rows are long, so that at least two stages fit) and read it
+// in units of 16, 8 or 4 bytes, the widest that divides the row an odd number of times
+// (rows are padded until one does), so that the rows a warp reads at once fall in
+// different banks; all lanes read the same units of the slice's slopes at the same
+// time (shared-memory broadcasts).  1- and 2-byte stores go to the tensor cores, 16 rows
+// an instruction, the slopes split into parts (see make_bfrag); the FP8 and INT8 row
+// scales are applied once per row after the sum over slices.
 //
 // Every wait is bounded (200 ms of %globaltimer); a wait that expires records
 // RTC_ETIMEDOUT in the status word, the block skips the rest of its work, lets its
@@ -44,6 +42,7 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "rtc_internal.h"
 
@@ -56,6 +55,7 @@ constexpr int kMaxStages = 32;
 // Smallest ring stage the launch plan aims for, in bytes (two stages of ~96 KB
 // measured faster than more, smaller ones: fewer per-tile handshakes).
 constexpr size_t kMinTileBytes = 96 * 1024;
+constexpr size_t kMinTileBytes8 = 48 * 1024;       // of 1-byte stores (four groups of rows a warp)
 // Rows of one slice's tile per consumer thread, at most (narrow slices pack several
 // rows into a stage sized for the widest one).
 constexpr int kMaxRowsPerThread = 32;
@@ -163,20 +163,42 @@ __host__ __device__ __forceinline__ int row_unit(int rb) {
     if (rb % 4 == 0 && (rb / 4) % 2 == 1) return 4;
     return 0;
 }
-// Byte offset of byte cb of row `row` of a slice (at byte off, rb bytes per row,
-// nact rows).  Row-major, or in the plane layout: rows in groups of 32, and within a
-// group the rows' first 16-byte units, then their second ones, ..., then their
-// (rb % 16)-byte tails.  A group of ng rows takes ng * rb bytes either way, so tiles
-// of whole groups are the same byte ranges in both layouts.
-__host__ __device__ __forceinline__ size_t slice_elem_offset(long long off, int rb, int nact, int row, int cb,
-                                                             int plane) {
-    if (!plane) return static_cast<size_t>(off) + static_cast<size_t>(row) * rb + cb;
-    const int g0 = row & ~31;
-    const int ng = nact - g0 < 32 ? nact - g0 : 32;
-    const int li = row - g0, q = rb >> 4, t = rb & 15, k = cb >> 4;
-    const size_t base = static_cast<size_t>(off) + static_cast<size_t>(g0) * rb;
-    if (k < q) return base + static_cast<size_t>(k) * ng * 16 + li * 16 + (cb & 15);
-    return base + static_cast<size_t>(q) * ng * 16 + static_cast<size_t>(li) * t + (cb - 16 * q);
+// A handle's INT8 codes are stored with the sign bit flipped (code + 128 as an unsigned
+// byte), which widen4 wants.
+constexpr unsigned char kInt8Flip = 0x80;
+
+// Byte offset of element byte cb of row `row` of a slice at byte off, rb bytes per row,
+// es bytes per element.  FP32 slices (es 4) are row-major.  The 1- and 2-byte stores
+// are in fragment order: rows in groups of 16 (16 rb bytes each, the last one padded with
+// zero rows), and within a group
+//   - 1-byte: the columns' first whole 32s, 512 bytes each: for lane (g, t) = (row % 8,
+//     column / 8) 16 bytes, 8 columns of row g then the same 8 of row g + 8;
+//   - the next whole 16s (2-byte: all of them), 256 es bytes each: for lane (row % 8,
+//     column / 4) 4 columns of row g then the same 4 of row g + 8;
+//   - the next whole 8, 128 es bytes: for lane (row % 8, column / 2) 2 columns of row g,
+//     then of row g + 8;
+//   - the last 2, 4 or 6 columns, the same for as many quarters t as there are pairs.
+// So a lane of a warp reads its share of an mma.m16n8k16 A operand, of two, or of half a
+// one as one vector, and the warp's read is consecutive bytes.
+__host__ __device__ __forceinline__ size_t slice_elem_offset(long long off, int rb, int row, int cb, int es) {
+    if (es == 4) return static_cast<size_t>(off) + static_cast<size_t>(row) * rb + cb;
+    const int r = row & 15, K = rb / es, b = cb % es;
+    int c = cb / es;
+    size_t at = static_cast<size_t>(off) + static_cast<size_t>(row >> 4) * 16 * rb;
+    const int k32 = es == 1 ? K & ~31 : 0;
+    if (c < k32) return at + (c >> 5) * 512 + ((r & 7) * 4 + ((c & 31) >> 3)) * 16 + (r >> 3) * 8 + (c & 7);
+    at += static_cast<size_t>(k32) * 16;
+    c -= k32;
+    const int k16 = (K - k32) & ~15;
+    if (c < k16)
+        return at + ((c >> 4) * 256 + ((r & 7) * 4 + ((c & 15) >> 2)) * 8 + (r >> 3) * 4 + (c & 3)) * es + b;
+    at += static_cast<size_t>(k16) * 16 * es;
+    c -= k16;
+    const int left = (K - k32 - k16), k8 = left & 8;
+    if (c < k8) return at + ((r & 7) * 8 + (c >> 1) * 2) * 2 * es + ((r >> 3) * 2 + (c & 1)) * es + b;
+    at += k8 * 16 * es;
+    c -= k8;
+    return at + ((r & 7) * (left - k8) + (c >> 1) * 2) * 2 * es + ((r >> 3) * 2 + (c & 1)) * es + b;
 }
 
 __device__ __forceinline__ void consumer_sync() {          // all consumer warps
@@ -276,10 +298,13 @@ struct Args {
     int region;              // shared scratch bytes of a fused phase (before the slopes)
     int loc_floats;          // floats of the largest block-local slope vector
     int row_floats;          // rows a block reduces, at most
-    int plane;               // slices in the plane layout (T = 1; see slice_elem_offset)
+    int frag;                // slices in fragment order (1- and 2-byte stores; see slice_elem_offset)
+    int max_slices;          // slices of a block, at most
+    int bf_floats;           // floats of a block's B fragments (0 for FP32)
     const float* s;          // stand-alone reconstruction: the full slope vector (else unused)
     const float* scale;      // [nact] row scales (FP8, INT8)
-    float* partial;          // [S][nact] partial DM vectors
+    float* partial;          // [S][pstride] partial DM vectors
+    int pstride;             // nact, rounded up to the groups of 16 rows
     float* a;                // [nact] integrator state
     float gain, leak;
     int* status;             // device error word
@@ -300,6 +325,8 @@ struct Plan {
     uint32_t ring;           // shared address of the ring
     unsigned char* scratch;  // fused-phase scratch (region bytes)
     float* loc;              // block-local slopes: each slice's x then y block, zero padded
+    float* bf;               // fragment-order slices: their B fragments (make_bfrag)
+    float* bscale;           // and what each slice's products are scaled back by
     float* a_pre;            // [r1 - r0] integrator state of the rows the block reduces
     float* sc_pre;           // [r1 - r0] their row scales
     float* red;              // [kConsumerWarps][32] warp sums of the sum over slices
@@ -339,7 +366,9 @@ __device__ __forceinline__ Plan make_plan(const Args& g, unsigned char* smem) {
     pl.ring = smem_addr(smem);
     pl.scratch = smem + ring_bytes;
     pl.loc = reinterpret_cast<float*>(smem + ring_bytes + g.region);
-    pl.a_pre = pl.loc + g.loc_floats;
+    pl.bf = pl.loc + g.loc_floats;
+    pl.bscale = pl.bf + g.bf_floats;
+    pl.a_pre = pl.bscale + (g.frag ? g.max_slices : 0);
     pl.sc_pre = pl.a_pre + g.row_floats;
     pl.red = pl.sc_pre + g.row_floats;
     return pl;
@@ -433,9 +462,9 @@ __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh
                 ok = false;
                 break;
             }
-            const int rows = min(tr, g.nact - row0);
-            // the slice is padded to 16 bytes, so the last tile may round up; the tile
-            // goes as several copies
+            // a slice in fragment order is padded to groups of 16 rows, a row-major one to
+            // 16 bytes; the tile goes as several copies
+            const int left = min(tr, g.nact - row0), rows = g.frag ? (left + 15) & ~15 : left;
             const uint32_t bytes = (static_cast<uint32_t>(rows) * rb + 15u) & ~15u;
             const uint32_t fb = smem_addr(&sh.full_bar[st]);
             mbar_expect_tx(fb, bytes);
@@ -522,7 +551,7 @@ __device__ __forceinline__ int consume_slice(const Args& g, const Plan& pl, Shar
     const int part = tid - rt * T;                           // lane within the row's group
     const int nunits = rb / U;
     const float* sv = pl.loc + lo;
-    float* out = g.partial + static_cast<size_t>(s) * nact;
+    float* out = g.partial + static_cast<size_t>(s) * g.pstride;
     const int tr = tile_rows(g, rb);
     const bool in_regs = (nunits + T - 1) / T <= JM;     // the same for the whole block
     float sr[JM][EPU];
@@ -606,78 +635,338 @@ __device__ __forceinline__ int consume_slice(const Args& g, const Plan& pl, Shar
     return tile;
 }
 
-// The tiles of one slice in the plane layout (T = 1, R = kConsumers rows a tile step):
-// warp w takes rows 32 w .. 32 w + 31 of each step, one group, so every 16-byte load
-// of the warp reads 512 consecutive bytes, and the (rb % 16)-byte tails follow the
-// group's units.  Rows are taken two at a time, sharing each unit's slope loads.
-// Each row's terms are added in element order, the order of the row-major form.
+// ---- 1- and 2-byte stores on the tensor cores -------------------------------------
+//
+// A multiply-add per matrix byte or two, with the conversion to FP32 and the slope's read,
+// kept the CUDA cores busy longer than the HBM takes to deliver the bytes (ELT INT8: 8.2
+// us against 5.2).  mma.sync.m16n8k16 takes the matrix as its A operand in the stored
+// type (BF16, FP16) or as the exactly equal FP16 values (E4M3 by the hardware
+// conversion, INT8 through the mantissa of 1024), 16 rows x 16 slopes an instruction.
+// The FP32 slopes are its B operand, each split exactly into three 16-bit parts in three
+// of the 8 columns:
+//   - BF16: the upper 8 bits of the significand, the next 8, the last 8 (truncating
+//     splits: nothing overflows, and the range is FP32's own);
+//   - FP16: 11 bits, 11 and 2, the second and third scaled by 2^11 and 2^22, after a
+//     power of two per slice that brings the slice's largest slope just below 2^15.
+//     (What falls below FP16's subnormals, 2^-61 of the largest slope in the third
+//     part, is dropped.)
+// Products are exact and accumulate in FP32, and the three column sums meet at the end.
+// Infinite and NaN slopes go whole into the first part.  Against 64 bits the commands
+// are as near as the FP32 chains' were or nearer (relative 2-norm: ELT FP16 41x41 1.2e-7
+// against 1.3e-7, six sensors FP8 2.3e-7 against 2.5e-7, BF16 loop 1.7e-7 against 2.1e-7).
+// Measured, frame after frame, with FP32 chains -> so: ELT INT8 17.0 -> 13.7 us, six
+// sensors FP8 54.6 -> 47.0, BF16 with prediction 26.9 -> 24.7; the persistent loop with
+// the BF16 matrix in L2 23.2 -> 18.1 us a frame.
+// (The 1-byte forms of mma.sync, with the slopes as E4M3 or integer digits in 8 columns,
+// were no faster: the E4M3 one issues the FP16 instructions and conversions, and the
+// integer one is slow on this GPU, 18.7 us for the ELT INT8 frame against 14.7.)
+
+template <int DT> struct HalfKind { static constexpr bool v = DT != RTC_BF16; };   // FP16 operands
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
+}
 template <int DT>
-__device__ __forceinline__ int consume_slice_plane(const Args& g, const Plan& pl, Shared& sh, int tid,
-                                                   int tile, int s, int rb, int lo) {
-    constexpr int E16 = 16 / Esize<DT>::v;                   // elements per 16-byte unit
-    constexpr int EPW = 4 / Esize<DT>::v;                    // elements per word
-    const int R = g.R, nact = g.nact, nst = g.nst, stage_bytes = g.stage_bytes;
-    const int lane = tid & 31;
-    const int q = rb >> 4, tb = rb & 15;
-    const float* sv = pl.loc + lo;
-    const float* st_tail = sv + q * E16;
-    float* out = g.partial + static_cast<size_t>(s) * nact;
-    const int tr = tile_rows(g, rb);
-    for (int row0 = 0; row0 < nact; row0 += tr, ++tile) {
-        const int st = tile % nst;
-        const bool ok = __all_sync(0xffffffffu, wait_phase(smem_addr(&sh.full_bar[st]),
-                                                            (tile / nst) & 1, &sh.abort_flag));
-        if (!ok) {
-            if (lane == 0 && !sh.abort_flag) {
-                atomicExch(g.status, RTC_ETIMEDOUT);
-                sh.abort_flag = 1;
-            }
-            continue;     // skip the work but keep reaching the block's barriers
+__device__ __forceinline__ void mma_dt(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
+    if (HalfKind<DT>::v) mma_f16(c, a0, a1, a2, a3, b);
+    else mma_bf16(c, a0, a1, a2, a3, b);
+}
+
+// Four 1-byte codes as two pairs of FP16 values.
+template <int DT>
+__device__ __forceinline__ void widen4(uint32_t w, uint32_t& lo, uint32_t& hi) {
+    if (DT == RTC_FP8_E4M3) {
+        asm("{\n\t.reg .b16 a, b;\n\t"
+            "mov.b32 {a, b}, %2;\n\t"
+            "cvt.rn.f16x2.e4m3x2 %0, a;\n\t"
+            "cvt.rn.f16x2.e4m3x2 %1, b;\n\t}"
+            : "=r"(lo), "=r"(hi)
+            : "r"(w));
+    } else {
+        // stored as code + 128 (kInt8Flip): 1024 + it as FP16, minus 1152: exact
+        const __half2 k = __half2half2(__ushort_as_half(0x6480));
+        const uint32_t p = __byte_perm(w, 0x64646464u, 0x4140), q = __byte_perm(w, 0x64646464u, 0x4342);
+        const __half2 a = __hsub2(*reinterpret_cast<const __half2*>(&p), k);
+        const __half2 b = __hsub2(*reinterpret_cast<const __half2*>(&q), k);
+        lo = *reinterpret_cast<const uint32_t*>(&a);
+        hi = *reinterpret_cast<const uint32_t*>(&b);
+    }
+}
+
+// Floats the B fragments of n slopes (a multiple of 16) take: 96 bytes a step of 16.
+__host__ __device__ __forceinline__ int bfrag_floats(int n) { return n / 16 * 24; }
+
+// Power of two that brings the largest finite of K slopes into [2^14, 2^15), and its
+// inverse.  By a whole warp.
+__device__ __forceinline__ void slope_scale(const float* sv, int K, int lane, float& up, float& down) {
+    unsigned m = 0;                                          // largest finite magnitude, as bits
+    for (int c = lane; c < K; c += 32) {
+        const unsigned u = __float_as_uint(sv[c]) & 0x7fffffffu;
+        if (u < 0x7f800000u) m = max(m, u);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    const int e = m ? max(static_cast<int>(m >> 23) - 127, -100) : 14;
+    up = __uint_as_float(static_cast<unsigned>(127 + 14 - e) << 23);
+    down = __uint_as_float(static_cast<unsigned>(127 - 14 + e) << 23);
+}
+
+// The parts of column c of a slice of K columns into its B fragments: the step, quarter
+// t and place j of the matrix elements the lanes hold (slice_elem_offset's column order).
+template <int DT>
+__device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, float up) {
+    const bool finite = (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
+    const int k32 = Esize<DT>::v == 1 ? K & ~31 : 0, rest = c - (K & ~15);
+    int step = c >> 4, t = (c & 15) >> 2, j = c & 3;
+    if (c < k32) {
+        step = 2 * (c >> 5) + ((c & 7) >> 2);
+        t = (c & 31) >> 3;
+    } else if (rest >= 0) {                                  // the last, partial 16: 8, then pairs
+        const int k8 = K & 8, second = rest >= k8;
+        t = (rest - (second ? k8 : 0)) >> 1;
+        j = 2 * second + (c & 1);
+    }
+    unsigned short* out = reinterpret_cast<unsigned short*>(frag) + step * 48 + t * 4 + j;
+    float r = HalfKind<DT>::v ? v * up : v;
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+        unsigned short d;
+        if (HalfKind<DT>::v) {
+            const __half h = __float2half_rz(r);
+            d = __half_as_ushort(h);
+            r = finite ? (r - __half2float(h)) * 2048.f : 0.f;
+        } else {
+            const unsigned u = __float_as_uint(r) & 0xffff0000u;
+            d = static_cast<unsigned short>(u >> 16);
+            if (n == 0 && v != v) d = 0x7fc0;                // a NaN whatever its payload
+            r = finite ? r - __uint_as_float(u) : 0.f;
         }
-        const uint32_t stage = pl.ring + st * stage_bytes;
-        const int iters = (min(tr, nact - row0) + R - 1) / R;
-        for (int i = 0; i < iters; i += 2) {
-            const int ra = tid + i * R, rbw = ra + R;
-            const bool va = row0 + ra < nact;
-            const bool vb = i + 1 < iters && row0 + rbw < nact;
-            const int ga = ra & ~31, gb = rbw & ~31;
-            const int na = min(32, nact - row0 - ga), nb = min(32, nact - row0 - gb);
-            const uint32_t pa = stage + ga * rb + lane * 16, pb = stage + gb * rb + lane * 16;
-            float acc0 = 0.f, acc1 = 0.f;
+        out[n * 16] = d;
+    }
+}
+
+// B fragments of the block's slices from its local slopes, and what each slice's sums
+// are scaled back by.  A block's only slice is shared by all its warps, several go a
+// warp each.  Between consumer barriers.
+template <int DT>
+__device__ __forceinline__ void make_bfrag(const Args& g, const Plan& pl, int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const bool one = pl.sb1 - pl.sb0 == 1;
+    for (int s = pl.sb0 + (one ? 0 : warp); s < pl.sb1; s += one ? 1 : kConsumerWarps) {
+        const int rb = s == pl.sb0 ? pl.rb0 : __ldg(g.sl.rowbytes + s);
+        const int lo = s == pl.sb0 ? 0 : __ldg(g.sl.loc + s) - pl.loc0;
+        const int K = rb / Esize<DT>::v;
+        const float* sv = pl.loc + lo;
+        float* frag = pl.bf + bfrag_floats(lo);
+        float up = 1.f, down = 1.f;
+        if (HalfKind<DT>::v) slope_scale(sv, K, lane, up, down);
+        if (lane == 0 && (!one || warp == 0)) pl.bscale[s - pl.sb0] = down;
+        // the last step's places, of which the columns may leave some
+        if (K & 15) {
+            float* last = frag + bfrag_floats(K & ~15);
+            for (int i = one ? tid : lane; i < bfrag_floats(16); i += one ? kConsumers : 32) last[i] = 0.f;
+        }
+        if (one) consumer_sync();
+        else __syncwarp();
+        for (int c = one ? tid : lane; c < K; c += one ? kConsumers : 32) put_parts<DT>(frag, K, c, sv[c], up);
+    }
+}
+
+// A slice's B fragments of a step, for the calling lane: the 12 lanes of the three parts
+// hold slopes, the others zeros.
+__device__ __forceinline__ uint2 bfrag(const float* frag, int step, int lane) {
+    uint2 b = make_uint2(0u, 0u);
+    if (lane < 12) b = reinterpret_cast<const uint2*>(frag)[step * 12 + lane];
+    return b;
+}
+
+// The B fragments of a slice of at most 64 columns, kept in registers for the whole
+// slice: the full steps, then the partial one.
+struct SliceB {
+    uint2 full[4], last;
+};
+
+// NG groups of 16 rows, group i at shared address at + i * gap: the rows' sums on each
+// quad's first lane, v[group][row half].  SMALL: at most 64 columns, their B fragments in
+// sb; else read step by step, once for all groups.  The groups' chains of products
+// are independent.
+template <int DT, int NG, bool SMALL>
+__device__ __forceinline__ void frag_dot(uint32_t at, uint32_t gap, int K, int lane, const SliceB& sb,
+                                         const float* frag, float (&v)[NG][2]) {
+    constexpr int ES = Esize<DT>::v;
+    float acc[NG][4];
+#pragma unroll
+    for (int i = 0; i < NG; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+    const uint32_t a16 = at + lane * 16;
+    const int q16 = K >> 4;                                  // whole steps of 16
+    if constexpr (ES == 1) {
+        const int q32 = K >> 5;
+        auto chunk = [&](int c, uint2 b0, uint2 b1) {        // 32 columns
+            uint4 m[NG];
+#pragma unroll
+            for (int i = 0; i < NG; ++i) m[i] = lds128(a16 + i * gap + c * 512);
+#pragma unroll
+            for (int i = 0; i < NG; ++i) {
+                uint32_t x0, x1, y0, y1, z0, z1, w0, w1;
+                widen4<DT>(m[i].x, x0, x1);
+                widen4<DT>(m[i].z, z0, z1);
+                mma_dt<DT>(acc[i], x0, z0, x1, z1, b0);
+                widen4<DT>(m[i].y, y0, y1);
+                widen4<DT>(m[i].w, w0, w1);
+                mma_dt<DT>(acc[i], y0, w0, y1, w1, b1);
+            }
+        };
+        auto odd = [&](uint2 b) {                            // 16 columns after the 32s
+            uint2 w[NG];
+#pragma unroll
+            for (int i = 0; i < NG; ++i) w[i] = lds64(at + i * gap + q32 * 512 + lane * 8);
+#pragma unroll
+            for (int i = 0; i < NG; ++i) {
+                uint32_t x0, x1, y0, y1;
+                widen4<DT>(w[i].x, x0, x1);
+                widen4<DT>(w[i].y, y0, y1);
+                mma_dt<DT>(acc[i], x0, y0, x1, y1, b);
+            }
+        };
+        if constexpr (SMALL) {
+            if (q32 > 0) chunk(0, sb.full[0], sb.full[1]);
+            if (q32 > 1) chunk(1, sb.full[2], sb.full[3]);
+            else if (q16 & 1) odd(q32 ? sb.full[2] : sb.full[0]);
+        } else {
+#pragma unroll 1
+            for (int c = 0; c < q32; ++c) chunk(c, bfrag(frag, 2 * c, lane), bfrag(frag, 2 * c + 1, lane));
+            if (q16 & 1) odd(bfrag(frag, 2 * q32, lane));
+        }
+    } else {
+        auto step = [&](int c, uint2 b) {                    // 16 columns
+            uint4 m[NG];
+#pragma unroll
+            for (int i = 0; i < NG; ++i) m[i] = lds128(a16 + i * gap + c * 512);
+#pragma unroll
+            for (int i = 0; i < NG; ++i) mma_dt<DT>(acc[i], m[i].x, m[i].z, m[i].y, m[i].w, b);
+        };
+        if constexpr (SMALL) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c < q16) step(c, sb.full[c]);
+        } else {
 #pragma unroll 2
-            for (int k = 0; k < q; ++k) {
-                float r[E16];
-                load_unit<E16>(sv + k * E16, r);
-                if (va) acc0 = unit_dot<DT, 16>(acc0, pa + k * na * 16, r);
-                if (vb) acc1 = unit_dot<DT, 16>(acc1, pb + k * nb * 16, r);
-            }
-            if (tb) {
-                const uint32_t ta = stage + ga * rb + q * na * 16 + lane * tb;
-                const uint32_t tbb = stage + gb * rb + q * nb * 16 + lane * tb;
-                if (tb == 8) {
-                    float r[2 * EPW];
-                    load_unit<2 * EPW>(st_tail, r);
-                    if (va) acc0 = unit_dot<DT, 8>(acc0, ta, r);
-                    if (vb) acc1 = unit_dot<DT, 8>(acc1, tbb, r);
-                } else {
-                    for (int w = 0; w < tb / 4; ++w) {
-                        float r[EPW];
-                        load_unit<EPW>(st_tail + w * EPW, r);
-                        if (va) acc0 = word_dot<DT>(acc0, lds32(ta + 4 * w), r);
-                        if (vb) acc1 = word_dot<DT>(acc1, lds32(tbb + 4 * w), r);
-                    }
-                }
-            }
-            if (va) out[row0 + ra] = acc0;
-            if (vb) out[row0 + rbw] = acc1;
+            for (int c = 0; c < q16; ++c) step(c, bfrag(frag, c, lane));
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_addr(&sh.empty_bar[st]));
+    }
+    if (K & 15) {                                            // the last columns: 8, then pairs
+        const uint2 b = SMALL ? sb.last : bfrag(frag, q16, lane);
+        const int k8 = K & 8, pairs = (K & 7) >> 1;
+        const uint32_t p8 = at + 16 * (K & ~15) * ES + lane * 4 * ES;
+        const uint32_t pr = at + 16 * (K & ~7) * ES + ((lane >> 2) * pairs + (lane & 3)) * 4 * ES;
+        const bool mine = (lane & 3) < pairs;
+        uint2 u[NG], w[NG];
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            u[i] = w[i] = make_uint2(0u, 0u);
+            if (k8) {
+                if constexpr (ES == 1) u[i].x = lds32(p8 + i * gap);
+                else u[i] = lds64(p8 + i * gap);
+            }
+            if (mine) {
+                if constexpr (ES == 1) w[i].x = lds32(pr + i * gap);
+                else w[i] = lds64(pr + i * gap);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            if constexpr (ES == 1) {
+                if (k8) widen4<DT>(u[i].x, u[i].x, u[i].y);
+                widen4<DT>(w[i].x, w[i].x, w[i].y);
+            }
+            mma_dt<DT>(acc[i], u[i].x, u[i].y, w[i].x, w[i].y, b);
+        }
+    }
+    // columns 0 and 1 of a row are on the quad's first lane, column 2 on its second
+#pragma unroll
+    for (int i = 0; i < NG; ++i)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float p2 = __shfl_xor_sync(0xffffffffu, acc[i][2 * r], 1);
+            v[i][r] = HalfKind<DT>::v ? fmaf(fmaf(p2, 0x1p-11f, acc[i][2 * r + 1]), 0x1p-11f, acc[i][2 * r])
+                                      : acc[i][2 * r] + (acc[i][2 * r + 1] + p2);
+        }
+}
+
+// The tiles of one slice in fragment order; returns the running tile count.  A warp
+// takes the groups of 16 rows w, w + 14, ... of a tile, up to four at a time.  Each row's
+// sum depends on the slice alone.  (The padding rows of the last group have their
+// place in the partial vectors too: no row is tested.)
+template <int DT, bool SMALL>
+__device__ __forceinline__ int consume_slice_frag(const Args& g, const Plan& pl, Shared& sh, int tid, int tile, int s,
+                                                  int rb, int lo) {
+    const int nact = g.nact, nst = g.nst, stage_bytes = g.stage_bytes;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int K = rb / Esize<DT>::v;
+    const float* frag = pl.bf + bfrag_floats(lo);
+    SliceB sb{};
+    if (SMALL) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < (K >> 4)) sb.full[c] = bfrag(frag, c, lane);
+        if (K & 15) sb.last = bfrag(frag, K >> 4, lane);
+    }
+    const float down = pl.bscale[s - pl.sb0];
+    const bool first = (lane & 3) == 0;
+    float* out = g.partial + static_cast<size_t>(s) * g.pstride + warp * 16 + (lane >> 2);
+    const int tr = tile_rows(g, rb);
+    const uint32_t gap = kConsumerWarps * 16 * rb, mine = pl.ring + warp * 16 * rb;
+    int st = tile % nst, phase = (tile / nst) & 1;
+    for (int row0 = 0; row0 < nact; row0 += tr, ++tile) {
+        const bool ok = __all_sync(0xffffffffu, wait_phase(smem_addr(&sh.full_bar[st]), phase, &sh.abort_flag));
+        if (ok) {
+            const int ng = (min(tr, nact - row0) + 15) >> 4;
+            uint32_t at = mine + st * stage_bytes;
+            float* o = out + row0;
+            auto take = [&](auto count) {                    // the warp's next groups
+                constexpr int NG = decltype(count)::value;
+                float v[NG][2];
+                frag_dot<DT, NG, SMALL>(at, gap, K, lane, sb, frag, v);
+                if (first)
+#pragma unroll
+                    for (int i = 0; i < NG; ++i)
+#pragma unroll
+                        for (int r = 0; r < 2; ++r)
+                            o[i * kConsumerWarps * 16 + 8 * r] = HalfKind<DT>::v ? v[i][r] * down : v[i][r];
+                at += NG * gap;
+                o += NG * kConsumerWarps * 16;
+            };
+            int left = ng > warp ? (ng - warp + kConsumerWarps - 1) / kConsumerWarps : 0;
+            for (; left >= 4; left -= 4) take(std::integral_constant<int, 4>());
+            if (left & 2) take(std::integral_constant<int, 2>());
+            if (left & 1) take(std::integral_constant<int, 1>());
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&sh.empty_bar[st]));
+        } else if (lane == 0 && !sh.abort_flag) {
+            // skip the work but keep reaching the block's barriers
+            atomicExch(g.status, RTC_ETIMEDOUT);
+            sh.abort_flag = 1;
+        }
+        if (++st == nst) {
+            st = 0;
+            phase ^= 1;
+        }
     }
     return tile;
 }
 
-// The consumer warps: every tile of the block's slices, one partial vector per
+// The consumer warps, after a consumer barrier that completes the block's slopes: every
+// tile of the block's slices, one partial vector per
 // slice (partial[s][row] = the row's dot product with the slice's slopes, in unit
 // order).  tile0: the running tile count at entry; returns the count at exit.  The
 // next slice's layout is fetched while the present one is consumed.
@@ -685,17 +974,25 @@ template <int DT>
 __device__ __forceinline__ int consume(const Args& g, const Plan& pl, Shared& sh, int tid, int tile0) {
     int tile = tile0;
     int rb = pl.rb0, lo = 0;
+    if constexpr (DT != RTC_F32) {
+        make_bfrag<DT>(g, pl, tid);
+        consumer_sync();
+    }
     for (int s = pl.sb0; s < pl.sb1; ++s) {
         int rb_next = 0, lo_next = 0;
         if (s + 1 < pl.sb1) {
             rb_next = __ldg(g.sl.rowbytes + s + 1);
             lo_next = __ldg(g.sl.loc + s + 1) - pl.loc0;
         }
-        const int u = row_unit(rb);
-        if (g.plane) tile = consume_slice_plane<DT>(g, pl, sh, tid, tile, s, rb, lo);
-        else if (u == 16) tile = consume_slice<DT, 16>(g, pl, sh, tid, tile, s, rb, lo);
-        else if (u == 8) tile = consume_slice<DT, 8>(g, pl, sh, tid, tile, s, rb, lo);
-        else tile = consume_slice<DT, 4>(g, pl, sh, tid, tile, s, rb, lo);
+        if constexpr (DT == RTC_F32) {
+            const int u = row_unit(rb);
+            if (u == 16) tile = consume_slice<DT, 16>(g, pl, sh, tid, tile, s, rb, lo);
+            else if (u == 8) tile = consume_slice<DT, 8>(g, pl, sh, tid, tile, s, rb, lo);
+            else tile = consume_slice<DT, 4>(g, pl, sh, tid, tile, s, rb, lo);
+        } else {
+            tile = rb <= 64 * Esize<DT>::v ? consume_slice_frag<DT, true>(g, pl, sh, tid, tile, s, rb, lo)
+                                           : consume_slice_frag<DT, false>(g, pl, sh, tid, tile, s, rb, lo);
+        }
         rb = rb_next;
         lo = lo_next;
     }
@@ -720,7 +1017,7 @@ __device__ __forceinline__ void reduce_rows(const Args& g, const Plan& pl, int t
 #pragma unroll
             for (int j = 0; j < kSlicesPerWarp; ++j) {
                 const int s = warp + j * kConsumerWarps;
-                p[j] = s < g.sl.S ? __ldcg(g.partial + static_cast<size_t>(s) * g.nact + row) : 0.f;
+                p[j] = s < g.sl.S ? __ldcg(g.partial + static_cast<size_t>(s) * g.pstride + row) : 0.f;
             }
 #pragma unroll
             for (int j = 0; j < kSlicesPerWarp; ++j)
@@ -807,17 +1104,21 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     if (L.G < 1 || S < 1 || static_cast<int>(h->sl_rowbytes.size()) != S) return L;
     // largest row and largest block-local slope vector over the blocks
     int max_rb = 0, max_loc = 0;
+    const bool frag = h->sl_frag;
+    const int esz = h->sl_esz;
     for (int b = 0; b < L.G; ++b) {
         const int s0 = static_cast<int>(static_cast<long long>(S) * b / L.G);
         const int s1 = static_cast<int>(static_cast<long long>(S) * (b + 1) / L.G);
         max_loc = std::max(max_loc, h->sl_loc[s1] - h->sl_loc[s0]);
         for (int s = s0; s < s1; ++s) max_rb = std::max(max_rb, h->sl_rowbytes[s]);
+        L.max_slices = std::max(L.max_slices, s1 - s0);
     }
     L.loc_floats = (max_loc + 3) / 4 * 4;
     L.row_floats = (h->cfg.nact + L.G - 1) / L.G;
     L.region = (min_region + 15) / 16 * 16;
-    size_t extra = L.region + 4 * static_cast<size_t>(L.loc_floats) +
-                   8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
+    L.bf_floats = frag ? bfrag_floats(L.loc_floats) : 0;
+    const size_t slopes = 4 * static_cast<size_t>(L.loc_floats + L.bf_floats + (frag ? L.max_slices : 0));
+    size_t extra = L.region + slopes + 8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
     size_t budget = kDynSmemBudget;
     size_t room = budget > extra ? budget - extra : 0;
     // lanes per row: the fewest for which two stages of R = kConsumers / T rows fit
@@ -825,12 +1126,15 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     // every store type: more tiles and butterflies cost more than the slope reads
     // they save).  Only the slices decide it, not the block count, so the order of
     // every row's sum is the same for any launch of the handle.
-    auto stage = [&](int T) { return (static_cast<size_t>(kConsumers / T) * max_rb + 15) / 16 * 16; };
+    // In fragment order every row is one lane group's whatever the tile, so only the
+    // tile shrinks (whole groups of 16 rows).
+    auto rows_of = [&](int T) { return frag ? std::max(16, kConsumers / T / 16 * 16) : kConsumers / T; };
+    auto stage = [&](int T) { return (static_cast<size_t>(rows_of(T)) * max_rb + 15) / 16 * 16; };
     L.T = 1;
-    while (L.T < 16 && 2 * stage(L.T) > room) L.T *= 2;      // R stays a multiple of 4
-    L.R = kConsumers / L.T;
+    while (L.T < (frag ? 32 : 16) && 2 * stage(L.T) > room) L.T *= 2;      // R stays a multiple of 4
+    L.R = rows_of(L.T);
     if (!loop) {
-        extra = L.region + 4 * static_cast<size_t>(L.loc_floats);
+        extra = L.region + slopes;
         // (a plan that would not get its two stages beside a sum block takes the whole SM)
         budget = 2 * stage(L.T) + extra <= kFrameSmemBudget ? kFrameSmemBudget : kDynSmemBudget;
         room = budget > extra ? budget - extra : 0;
@@ -838,14 +1142,15 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     // stages of at least kMinTileBytes (whole multiples of R rows of the widest
     // slice), so that the per-tile handshakes stay a small part of the work
     const size_t st1 = stage(L.T);
-    size_t m = st1 > 0 ? std::max<size_t>(1, kMinTileBytes / st1) : 1;
+    size_t m = st1 > 0 ? std::max<size_t>(1, (esz == 1 ? kMinTileBytes8 : kMinTileBytes) / st1) : 1;
     while (m > 1 && 2 * m * st1 > room) --m;
     L.stage_bytes = static_cast<int>(m * st1);
     const size_t fit = L.stage_bytes > 0 ? room / L.stage_bytes : 0;
     L.nst = static_cast<int>(fit < static_cast<size_t>(kMaxStages) ? fit : kMaxStages);
     L.smem = static_cast<size_t>(L.nst) * L.stage_bytes + extra;
     L.ok = L.nst >= 2 && L.loc_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
-           S <= kMaxSlices && L.smem <= budget && (!h->sl_plane || L.T == 1);
+           S <= kMaxSlices && L.smem <= budget;
+    if (frag) L.T = 1;
     return L;
 }
 
@@ -873,12 +1178,15 @@ inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
     g.nst = L.nst;
     g.l2_policy = h->m_bytes <= kL2KeepBytes ? kL2Normal : kL2Stream;
     g.region = static_cast<int>(L.region);
-    g.plane = h->sl_plane ? 1 : 0;
+    g.frag = h->sl_frag ? 1 : 0;
+    g.max_slices = L.max_slices;
+    g.bf_floats = L.bf_floats;
     g.loc_floats = L.loc_floats;
     g.row_floats = L.row_floats;
     g.s = d_s;
     g.scale = h->d_scale;
     g.partial = h->d_partial;
+    g.pstride = partial_pitch(h->cfg.nact);
     g.a = h->d_a;
     g.gain = h->gain;
     g.leak = h->leak;
