@@ -13,8 +13,7 @@
 struct rtc_mlp {
     int device = 0;
     MlpDev w{};
-    float* parts = nullptr;      // [nparts_cap][kMlpPartPitch] block partials
-    int nparts_cap = 0;
+    float* parts = nullptr;      // [sms][kMlpPartPitch] block partials, for any batch size
     int* d_nbr = nullptr;        // [nv][25] neighbour table (rtc_mlp_set_geometry)
     int nv = 0;
     int step = 0;                // Adam steps taken
@@ -39,18 +38,6 @@ struct Dev {
         if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
     }
 };
-
-int ensure_parts(rtc_mlp* m, int B) {
-    const int need = mlp_blocks(B, m->sms);
-    if (need <= m->nparts_cap) return RTC_OK;
-    if (m->parts) cudaFree(m->parts);
-    m->parts = nullptr;
-    m->nparts_cap = 0;
-    if (cudaMalloc(&m->parts, static_cast<size_t>(need) * kMlpPartPitch * sizeof(float)) != cudaSuccess)
-        return mfail(RTC_ENOMEM, "cannot allocate the gradient partials");
-    m->nparts_cap = need;
-    return RTC_OK;
-}
 
 }  // namespace
 
@@ -121,7 +108,9 @@ int rtc_mlp_create(int32_t device, rtc_mlp** out) {
     rtc_mlp* m = new rtc_mlp();
     m->device = device;
     cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, device);
-    const int rc = mlp_alloc(m->w);
+    int rc = mlp_alloc(m->w);
+    if (rc == RTC_OK && cudaMalloc(&m->parts, static_cast<size_t>(m->sms) * kMlpPartPitch * sizeof(float)) != cudaSuccess)
+        rc = RTC_ENOMEM;
     if (rc != RTC_OK) {
         mlp_free(m->w);
         delete m;
@@ -194,8 +183,6 @@ int rtc_mlp_gradient(rtc_mlp* m, const float* d_X, const float* d_T, int32_t B, 
                      float* d_loss, void* stream) {
     if (!m || B <= 0 || !d_X || !d_T || !d_grad) return mfail(RTC_EINVAL, "bad arguments");
     Dev d(m->device);
-    int rc = ensure_parts(m, B);
-    if (rc != RTC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, mlp_blocks(B, m->sms), st) != cudaSuccess ||
         mlp_launch_update(m->w, m->parts, mlp_blocks(B, m->sms), B, 0.f, 0.9f, 0.999f, 1e-8f, 1,
@@ -208,8 +195,6 @@ int rtc_mlp_train_step(rtc_mlp* m, const float* d_X, const float* d_T, int32_t B
                        float* d_loss, void* stream) {
     if (!m || B <= 0 || !d_X || !d_T || !(lr > 0.f)) return mfail(RTC_EINVAL, "bad arguments");
     Dev d(m->device);
-    int rc = ensure_parts(m, B);
-    if (rc != RTC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     m->step += 1;
     if (mlp_launch_train(m->w, d_X, d_T, B, m->parts, mlp_blocks(B, m->sms), st) != cudaSuccess ||
@@ -225,8 +210,6 @@ int rtc_mlp_train_seq(rtc_mlp* m, const float* d_S, int32_t n_frames, const int3
         return mfail(RTC_EINVAL, "bad arguments");
     if (!m->d_nbr) return mfail(RTC_ESTATE, "rtc_mlp_set_geometry first");
     Dev d(m->device);
-    int rc = ensure_parts(m, B);
-    if (rc != RTC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     m->step += 1;
     if (mlp_launch_train_seq(m->w, d_S, n_frames, m->nv, m->d_nbr,
