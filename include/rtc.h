@@ -457,7 +457,7 @@ int rtc_mlp_predict_seq(rtc_mlp* m, const float* d_S, int32_t n_frames, float si
 int rtc_load_predictor(rtc_handle* h, const float* params, int64_t n, float sigma);
 int rtc_set_predictor(rtc_handle* h, int32_t on);
 
-/* Largest sizes rtc_mvm_integrate_noalloc accepts (its scratch is fixed at load). */
+/* Largest sizes rtc_mvm_integrate_noalloc accepts. */
 #define RTC_NOALLOC_MAX_NACT   8192
 #define RTC_NOALLOC_MAX_KSPLIT 16
 
@@ -467,9 +467,7 @@ int rtc_set_predictor(rtc_handle* h, int32_t on);
  * which cannot afford the implicit device synchronisation and unbounded latency
  * of cudaMalloc inside its loop, or a plugin inside a larger RTC framework that
  * receives every device buffer from the framework and may not allocate its own.
- * It needs no handle and allocates nothing: the split-K scratch lives in a
- * static device array of about 520 KiB, held by every GPU that loads the library
- * until the process exits.
+ * It needs no handle, allocates nothing and keeps no scratch in device memory.
  *
  * Buffers (all device memory on the current device, owned by the caller):
  *   d_M          [nact][kpad] matrix in the stored type `store` (rtc_dtype),
@@ -484,12 +482,12 @@ int rtc_set_predictor(rtc_handle* h, int32_t on);
  * The work is enqueued on `stream` (a cudaStream_t; NULL is the legacy default
  * stream) without synchronising.
  *
- * The first call on a device looks up the scratch array's device address (this
- * may load the library's device code); make that first call before any stream
- * capture.  Every call on a device shares the one scratch array, which keeps the
- * last call's contents; each call clears the counters it needs before its kernel.
- * Calls whose work overlaps on the GPU (unordered streams) race on the scratch
- * and give wrong results: order them on one stream.
+ * ksplit, the number of column splits, is accepted for callers that pass one; the
+ * result does not depend on it.
+ *
+ * The first call on a device configures the kernels (this may load the library's
+ * device code); make that first call before any stream capture.  Calls on different
+ * streams are independent (a call orders only its own buffers).
  * Errors: RTC_EINVAL, RTC_EDEVICE. */
 int rtc_mvm_integrate_noalloc(const void* d_M, int32_t store, const float* d_row_scales,
                               int32_t nact, int32_t kpad, const float* d_s, float* d_a,

@@ -11,13 +11,8 @@
 
 #include "rtc.h"
 
-// Threads per block of the pixel stage and of the reconstruction stage.
+// Threads per block of the pixel stage.
 constexpr int kCalibThreads = 256;
-constexpr int kMvmThreads = 256;
-// Matrix rows handled together by one reconstruction block.
-constexpr int kMvmRows = 4;
-// Largest split-K factor (partials per actuator summed by the fixed-order tree).
-constexpr int kMaxKsplit = 32;
 
 // Completion record of one loop frame, written by the device into mapped host memory.
 struct rtc_loop_done {
@@ -203,13 +198,6 @@ cudaError_t launch_frame(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out
                          int head, cudaStream_t st, FrameHost* fh = nullptr, float* d_s2 = nullptr);
 cudaError_t launch_mvm_integrate(rtc_handle* h, const float* d_s, float* d_dm_out,
                                  cudaStream_t st);
-
-// The same split-K MVM + integrator on caller-described buffers: matrix [nact][kpad]
-// in the stored type, s [kpad], partial scratch [ksplit][nact], counters
-// [ceil(nact/kMvmRows)] that must be zero on entry.
-cudaError_t launch_mvm_raw(int store, const void* d_M, const float* d_scale, int nact, int kpad,
-                           const float* d_s, int ksplit, float* d_partial, unsigned* d_count,
-                           float* d_a, float* d_dm_out, float gain, float leak, cudaStream_t st);
 
 // Store a device matrix [nact][ncol] (FP32, or already in the stored type when
 // src == store) into the slice-major layout: column c goes to slice colmap[c].x,
