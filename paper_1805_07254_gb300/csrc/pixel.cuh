@@ -175,6 +175,19 @@ __device__ __forceinline__ float2 subap_slopes_at(const PixelArgs& p, const uint
     return res;
 }
 
+// Brings the lines of one subaperture's pixel rows into L2, by an aligned group of 16
+// lanes.  Only a hint: it may run before the frame is written.
+__device__ __forceinline__ void prefetch_rows_l2(const PixelArgs& p, int gi, bool valid, int2 pos, int lane) {
+    if (!valid) return;
+    const uint16_t* box = p.frame + static_cast<size_t>(gi / p.n_valid) * p.side * p.side +
+                          static_cast<size_t>(pos.x) * p.npx * p.side + static_cast<size_t>(pos.y) * p.npx;
+    for (int y = lane & 15; y < p.npx; y += 16) {
+        const uint16_t* row = box + static_cast<size_t>(y) * p.side;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(row + p.npx - 1));
+    }
+}
+
 // ---- frame ingest from host memory ---------------------------------------------
 // A block copies exactly the pixel rows its subapertures cover from a frame in
 // mapped host memory into a device staging buffer, as a host-built, sorted list of

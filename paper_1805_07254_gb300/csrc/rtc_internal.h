@@ -63,7 +63,7 @@ inline int partial_pitch(int nact) { return (nact + 15) / 16 * 16; }
 
 // Grid, tiles, stages and dynamic shared memory of a streaming launch (stream_mvm.cuh).
 struct LaunchPlan {
-    int G, T, R, nst, stage_bytes, loc_floats, row_floats, max_slices, bf_floats;
+    int G, T, R, nst, stage_bytes, loc_floats, row_floats, max_slices, bf_floats, pre_tiles, l2_ahead;
     size_t smem, region;
     bool ok;
 };

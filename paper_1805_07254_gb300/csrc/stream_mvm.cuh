@@ -131,6 +131,10 @@ __device__ __forceinline__ unsigned long long matrix_policy(int mode) {
         asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
+// Bulk prefetch of global bytes into L2 (no shared memory, no completion).
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -299,6 +303,8 @@ struct Args {
     int loc_floats;          // floats of the largest block-local slope vector
     int row_floats;          // rows a block reduces, at most
     int frag;                // slices in fragment order (1- and 2-byte stores; see slice_elem_offset)
+    int pre_tiles;           // tiles requested before the previous kernel is complete
+    int l2_ahead;            // tiles brought into L2 once the ring has been requested
     int max_slices;          // slices of a block, at most
     int bf_floats;           // floats of a block's B fragments (0 for FP32)
     const float* s;          // stand-alone reconstruction: the full slope vector (else unused)
@@ -343,15 +349,19 @@ __device__ __forceinline__ void init_shared(Shared& sh) {
 
 __device__ __forceinline__ Plan make_plan(const Args& g, unsigned char* smem) {
     Plan pl;
-    const int S = g.sl.S;
-    pl.sb0 = static_cast<int>(static_cast<long long>(S) * blockIdx.x / gridDim.x);
-    pl.sb1 = static_cast<int>(static_cast<long long>(S) * (blockIdx.x + 1) / gridDim.x);
+    const unsigned S = g.sl.S;
+    // (32-bit products: a plan has at most 256 slices, and at most 4096 subapertures a slice
+    // and rows a block; a 64-bit division is some 80 instructions in every warp)
+    const unsigned b = blockIdx.x, G = gridDim.x;
+    pl.sb0 = S * b / G;
+    pl.sb1 = S * (b + 1) / G;
     // the block's subapertures: with the default cut computed, so that the pixel
     // stage does not wait for a table load before it can fetch positions
     if (g.sl.equal) {
-        pl.g0 = static_cast<int>(static_cast<long long>(g.sl.nt) * pl.sb0 / S);
-        pl.g1 = static_cast<int>(static_cast<long long>(g.sl.nt) * pl.sb1 / S);
-        pl.n0 = static_cast<int>(static_cast<long long>(g.sl.nt) * (pl.sb0 + 1) / S) - pl.g0;
+        const unsigned nt = g.sl.nt;
+        pl.g0 = nt * pl.sb0 / S;
+        pl.g1 = nt * pl.sb1 / S;
+        pl.n0 = nt * (pl.sb0 + 1) / S - pl.g0;
     } else {
         pl.g0 = g.sl.g0[pl.sb0];
         pl.g1 = g.sl.g0[pl.sb1];
@@ -360,8 +370,8 @@ __device__ __forceinline__ Plan make_plan(const Args& g, unsigned char* smem) {
     // the first slice's layout, read once here rather than on the frame's critical path
     pl.rb0 = g.sl.rowbytes[pl.sb0];
     pl.loc0 = g.sl.loc[pl.sb0];
-    pl.r0 = static_cast<int>(static_cast<long long>(g.nact) * blockIdx.x / gridDim.x);
-    pl.r1 = static_cast<int>(static_cast<long long>(g.nact) * (blockIdx.x + 1) / gridDim.x);
+    pl.r0 = static_cast<unsigned>(g.nact) * b / G;
+    pl.r1 = static_cast<unsigned>(g.nact) * (b + 1) / G;
     const int ring_bytes = g.nst * g.stage_bytes;
     pl.ring = smem_addr(smem);
     pl.scratch = smem + ring_bytes;
@@ -446,7 +456,9 @@ __device__ __forceinline__ int tile_rows(const Args& g, int rb) {
 // frame after frame in a persistent kernel); returns the count at exit.  drain: wait
 // for the last copies to land before returning (a block must not exit with copies
 // in flight).  The ring fills before the block's slopes are known and then waits for
-// its consumers.
+// its consumers.  A per-frame kernel requests its first pre_tiles tiles before its
+// predecessor is complete, the others after (the persistent loop has no predecessor),
+// and l2_ahead further ones into L2 (see Launch::pre_tiles).
 __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh, int tl0 = 0, bool drain = true) {
     int tl = tl0;
     bool ok = true;
@@ -456,6 +468,12 @@ __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh
         const int rb = g.sl.rowbytes[s];
         const int tr = tile_rows(g, rb);
         for (int row0 = 0; row0 < g.nact; row0 += tr, ++tl) {
+            if (tl == g.pre_tiles) asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (g.l2_ahead && tl == g.nst) {
+                const uint32_t ahead = (static_cast<uint32_t>(min(g.l2_ahead * tr, g.nact - row0)) * rb) & ~15u;
+                const unsigned char* next = base + static_cast<size_t>(row0) * rb;
+                for (uint32_t o = 0; o < ahead; o += kCopyBytes) bulk_prefetch_l2(next + o, min(kCopyBytes, ahead - o));
+            }
             const int st = tl % g.nst;
             const int use = tl / g.nst;
             if (use > 0 && !wait_phase(smem_addr(&sh.empty_bar[st]), (use - 1) & 1, &sh.abort_flag)) {
@@ -1091,7 +1109,19 @@ __device__ __forceinline__ void finish_host(const FrameHost& fh, const int* stat
     }
 }
 
+// How much of the matrix a per-frame kernel requests when.  Its blocks start while the
+// last frame's sum still has to read the partials and while their own pixels are not
+// there; matrix traffic then delays both, but later there is too little time for it:
+//   - the ring holds most of the block's share: nothing before the wait, since it fills
+//     during the pixel stage anyway (ELT INT8 13.3 us against 13.9 with one tile early
+//     and 14.1 with the whole ring; FP8 12.7, 13.2, 13.5);
+//   - it holds less than half: one tile early, the rest of the ring at the wait and two
+//     tiles more into L2, which the HBM fetches during the pixel stage (ELT FP32 23.7 us
+//     against 26.2 with the whole ring early and nothing ahead, BF16 15.9 against 17.4);
+//   - several pixel rounds a block (more sensors): the ring early and nothing ahead,
+//     the pixel stage itself takes the HBM (six sensors FP8 47.8 us against 50).
 using Launch = LaunchPlan;
+constexpr int kAllTiles = 1 << 30;
 
 // min_region: shared-memory scratch a fused phase needs.  loop: the persistent kernel,
 // which also sums its rows (integrator state, row scales and warp sums in shared
@@ -1148,6 +1178,12 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     const size_t fit = L.stage_bytes > 0 ? room / L.stage_bytes : 0;
     L.nst = static_cast<int>(fit < static_cast<size_t>(kMaxStages) ? fit : kMaxStages);
     L.smem = static_cast<size_t>(L.nst) * L.stage_bytes + extra;
+    L.pre_tiles = kAllTiles;
+    if (!loop && min_region == 0 && h->n_valid * static_cast<long long>(h->cfg.n_wfs) <= 2ll * kConsumerWarps * L.G) {
+        const bool most = 2ll * L.nst * L.stage_bytes * L.G >= h->m_bytes;
+        L.pre_tiles = most ? 0 : 1;
+        L.l2_ahead = most ? 0 : 2;
+    }
     L.ok = L.nst >= 2 && L.loc_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
            S <= kMaxSlices && L.smem <= budget;
     if (frag) L.T = 1;
@@ -1181,6 +1217,8 @@ inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
     g.frag = h->sl_frag ? 1 : 0;
     g.max_slices = L.max_slices;
     g.bf_floats = L.bf_floats;
+    g.pre_tiles = L.pre_tiles;
+    g.l2_ahead = L.l2_ahead;
     g.loc_floats = L.loc_floats;
     g.row_floats = L.row_floats;
     g.s = d_s;
