@@ -24,12 +24,15 @@
 // caller's completion record, so the host needs no copies and no stream
 // synchronisation.
 //
+// A small system's sum is done by the last streaming block instead (last_block_sum),
+// except for HOST frames.
+//
 // Measured, frame after frame on one stream (one cooperative kernel with a grid barrier
-// -> this): ELT FP32 28.9 -> 25.4 us, INT8 20.9 -> 17.0, BF16 with prediction 28.4 ->
-// 27.1, six ELT sensors FP8 59.4 -> 54.6, 41x41 FP16 12.3 -> 7.6 and 8x8 FP32 10.3 -> 6.2
-// (GPU time; the two launches' host time, 4 us in the library, bounds the last two).  Of
-// an FP32 frame the blocks stream 17 us (6.5 TB/s); slopes are known 2.9 us after the
-// last frame's sum, the hand-over to the sum takes 0.9 us and the sum 1.4.
+// -> this): ELT FP32 28.9 -> 23.1 us, INT8 20.9 -> 12.9, BF16 with prediction 28.4 ->
+// 25.0, six ELT sensors FP8 59.4 -> 47.4, 41x41 FP16 12.3 -> 7.9 of GPU time (9.2 with
+// the two launches' host time, which bounds it) and 8x8 FP32 10.3 -> 6.8.  Of an FP32
+// frame the blocks stream 17 us (6.5 TB/s); slopes are known 2.9 us after the last
+// frame's sum, the hand-over to the sum takes 0.9 us and the sum 1.4.
 
 #include "launch.cuh"
 #include "mlp.h"
@@ -74,9 +77,10 @@ __device__ __forceinline__ void pixel_stage(const rtc_pixel::PixelArgs& px, cons
     }
 }
 
-template <int DT, int NPX, bool HOST>
+// LAST: the last block also sums (last_block_sum), and the launch is the whole frame.
+template <int DT, int NPX, bool HOST, bool LAST>
 __global__ void __launch_bounds__(kFrameRegThreads, 1)
-frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh) {
+frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
@@ -98,6 +102,10 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh) {
     pdl_wait();                         // before the partials of the last frame are overwritten
     consumer_sync();
     consume<DT>(g, pl, sh, tid, 0);
+    if (LAST) {
+        __shared__ int last;
+        last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
+    }
 }
 
 // The pixel stage alone, for a frame in host memory and the predictor.
@@ -116,8 +124,9 @@ __global__ void __launch_bounds__(kThreads, 1) frame_slopes_kernel(rtc_pixel::Pi
 // the kernel before this one.  That kernel lets this one start at once, so that the ring
 // fills and the network's weights arrive while the pixel stage waits for the frame; the
 // history is read after the wait.
-template <int DT>
-__global__ void __launch_bounds__(kFrameRegThreads, 1) frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head) {
+template <int DT, bool LAST>
+__global__ void __launch_bounds__(kFrameRegThreads, 1)
+frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
@@ -145,14 +154,20 @@ __global__ void __launch_bounds__(kFrameRegThreads, 1) frame_pred_kernel(Args g,
         });
     consumer_sync();
     consume<DT>(g, pl, sh, tid, 0);
+    if (LAST) {
+        __shared__ int last;
+        last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
+    }
 }
 
-template <int DT, bool HOST>
+template <int DT, int NPX>
 cudaError_t launch_npx(const rtc_handle* h, const Launch& L, const rtc_pixel::PixelArgs& px, const Args& g,
-                       const FrameHost& fh, cudaStream_t st) {
+                       const FrameHost* fh, bool last, const SumArgs& sa, cudaStream_t st) {
     const dim3 grid(L.G), block(kThreads);
-    if (h->cfg.npx == 10) return launch_pdl(frame_kernel<DT, 10, HOST>, grid, block, L.smem, st, px, g, fh);
-    return launch_pdl(frame_kernel<DT, 0, HOST>, grid, block, L.smem, st, px, g, fh);
+    unsigned* ctr = h->d_lastctr;
+    if (fh) return launch_pdl(frame_kernel<DT, NPX, true, false>, grid, block, L.smem, st, px, g, *fh, sa, ctr);
+    if (last) return launch_pdl(frame_kernel<DT, NPX, false, true>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
+    return launch_pdl(frame_kernel<DT, NPX, false, false>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
 }
 
 template <int DT>
@@ -175,17 +190,21 @@ cudaError_t launch_dt(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, f
         fh->blk = h->d_blk;
         fh->stage = h->d_frame;
     }
+    const bool last = !fh && last_block_sums(h->sl_S, h->cfg.nact);
+    const SumArgs sa = last ? sum_args(h, d_dm_out) : SumArgs{};
+    const bool n10 = h->cfg.npx == 10;
     cudaError_t e;
     if (!pred) {
-        e = fh ? launch_npx<DT, true>(h, L, px, g, *fh, st) : launch_npx<DT, false>(h, L, px, g, FrameHost{}, st);
+        e = n10 ? launch_npx<DT, 10>(h, L, px, g, fh, last, sa, st) : launch_npx<DT, 0>(h, L, px, g, fh, last, sa, st);
     } else {
+        const dim3 grid(L.G), block(kThreads);
         if (!fh) e = launch_calib_cog(h, d_frame, d_s_meas, d_s2, true, st);
-        else if (h->cfg.npx == 10) e = launch_pdl(frame_slopes_kernel<10>, dim3(L.G), dim3(kThreads), 0, st, px, g, *fh);
-        else e = launch_pdl(frame_slopes_kernel<0>, dim3(L.G), dim3(kThreads), 0, st, px, g, *fh);
-        if (e == cudaSuccess)
-            e = launch_pdl(frame_pred_kernel<DT>, dim3(L.G), dim3(kThreads), L.smem, st, g, pred_args(h), head);
+        else if (n10) e = launch_pdl(frame_slopes_kernel<10>, grid, block, 0, st, px, g, *fh);
+        else e = launch_pdl(frame_slopes_kernel<0>, grid, block, 0, st, px, g, *fh);
+        const auto k = last ? frame_pred_kernel<DT, true> : frame_pred_kernel<DT, false>;
+        if (e == cudaSuccess) e = launch_pdl(k, grid, block, L.smem, st, g, pred_args(h), head, sa, h->d_lastctr);
     }
-    return e == cudaSuccess ? launch_sum(h, d_dm_out, st, fh) : e;
+    return e == cudaSuccess && !last ? launch_sum(h, d_dm_out, st, fh) : e;
 }
 
 template <typename K>
@@ -193,13 +212,20 @@ cudaError_t configure(K kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDynSmemBudget));
 }
 
+template <int DT, int NPX>
+cudaError_t configure_npx() {
+    cudaError_t e = configure(frame_kernel<DT, NPX, false, false>);
+    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, false, true>);
+    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, true, false>);
+    return e;
+}
+
 template <int DT>
 cudaError_t configure_dt() {
-    cudaError_t e = configure(frame_kernel<DT, 10, false>);
-    if (e == cudaSuccess) e = configure(frame_kernel<DT, 0, false>);
-    if (e == cudaSuccess) e = configure(frame_kernel<DT, 10, true>);
-    if (e == cudaSuccess) e = configure(frame_kernel<DT, 0, true>);
-    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT>);
+    cudaError_t e = configure_npx<DT, 10>();
+    if (e == cudaSuccess) e = configure_npx<DT, 0>();
+    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, false>);
+    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, true>);
     return e;
 }
 

@@ -49,16 +49,6 @@ __global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g)
 // 32 rows a block, one per lane; the order of reduce_rows (stream_mvm.cuh).  A step that
 // a bounded wait cut short (status) leaves the integrator as it was.  HOST: the last
 // block to finish writes the caller's completion record.
-struct SumArgs {
-    const float* partial;    // [S][pitch]
-    const float* scale;      // [nact] row scales, or null
-    float* a;
-    float* dm_out;           // [nact] or null
-    int* status;
-    int S, nact, pitch;
-    float gain, leak;
-};
-
 template <bool HOST>
 __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, FrameHost fh) {
     __shared__ float red[kConsumerWarps * 32];
@@ -139,10 +129,14 @@ cudaError_t configure_one() {
 
 }  // namespace
 
-cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {
+rtc_mvm::SumArgs sum_args(const rtc_handle* h, float* d_dm_out) {
     const bool scaled = h->store == RTC_FP8_E4M3 || h->store == RTC_INT8;
-    const SumArgs r{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a,  d_dm_out, h->d_status, h->sl_S,
-                    h->cfg.nact,  partial_pitch(h->cfg.nact),    h->gain, h->leak};
+    return SumArgs{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a,  d_dm_out, h->d_status, h->sl_S,
+                   h->cfg.nact,  partial_pitch(h->cfg.nact),    h->gain, h->leak};
+}
+
+cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {
+    const SumArgs r = sum_args(h, d_dm_out);
     const dim3 grid((h->cfg.nact + 31) / 32), block(kConsumers);
     if (!fh) return launch_pdl(mvm_reduce_kernel<false>, grid, block, 0, st, r, FrameHost{});
     fh->target = h->pf_arrivals + grid.x;

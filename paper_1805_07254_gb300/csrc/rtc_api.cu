@@ -472,11 +472,13 @@ int rtc_create(const rtc_config* cfg, rtc_handle** out) {
             cudaMalloc(&h->d_frame, frame_elems * sizeof(uint16_t)) != cudaSuccess ||
             cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess ||
             cudaMalloc(&h->d_gridbar, sizeof(unsigned long long)) != cudaSuccess ||
+            cudaMalloc(&h->d_lastctr, sizeof(unsigned)) != cudaSuccess ||
             cudaMallocHost(&h->h_status, sizeof(int)) != cudaSuccess) {
             rcode = fail(nullptr, RTC_ENOMEM, "device allocation failed");
         } else if (cudaMemset(h->d_a, 0, c.nact * sizeof(float)) != cudaSuccess ||
                    cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess ||
-                   cudaMemset(h->d_gridbar, 0, sizeof(unsigned long long)) != cudaSuccess) {
+                   cudaMemset(h->d_gridbar, 0, sizeof(unsigned long long)) != cudaSuccess ||
+                   cudaMemset(h->d_lastctr, 0, sizeof(unsigned)) != cudaSuccess) {
             rcode = fail(nullptr, RTC_EDEVICE, "cudaMemset failed");
         } else {
             rcode = apply_subaps(h, default_subaps(c.nsub, c.obs));
@@ -514,6 +516,7 @@ int rtc_destroy(rtc_handle* h) {
     free_dev(h->d_frame);
     free_dev(h->d_status);
     free_dev(h->d_gridbar);
+    free_dev(h->d_lastctr);
     free_dev(h->d_sbuf);
     free_dev(h->d_donectr);
     free_dev(h->d_mirror);

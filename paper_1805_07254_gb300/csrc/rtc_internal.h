@@ -119,6 +119,7 @@ struct rtc_handle {
     uint16_t* d_frame = nullptr;    // [n_wfs][side][side] staging for host frames
     int* d_status = nullptr;        // device-side error word (RTC_ETIMEDOUT from bounded waits)
     unsigned long long* d_gridbar = nullptr;  // grid-barrier arrival counter (only grows)
+    unsigned* d_lastctr = nullptr;            // finished blocks of a launch whose last block sums (wraps)
     unsigned long long grid_epoch = 0;        // block arrivals expected so far on d_gridbar
 
     // persistent loop (allocated by the first rtc_run_loop)

@@ -1059,6 +1059,87 @@ __device__ __forceinline__ void reduce_rows(const Args& g, const Plan& pl, int t
     }
 }
 
+// What the sum over slices and the integrator of a per-frame call need.
+struct SumArgs {
+    const float* partial;    // [S][pitch]
+    const float* scale;      // [nact] row scales, or null
+    float* a;
+    float* dm_out;           // [nact] or null
+    int* status;
+    int S, nact, pitch;
+    float gain, leak;
+};
+
+// Small systems: the whole sum by the last of the streaming blocks to finish, in its
+// ring (drained by then), instead of by a kernel of its own.  No block waits for another.
+// It takes 0.6 us longer on the GPU than the overlapped sum kernel at 4,000 values, but
+// saves a launch, 1.4 us of the host's time, which is what bounds such frames.  Measured
+// per frame in a stream of frames (two kernels -> this): 4,000 values (8x8) 9.0 -> 6.8 us,
+// with prediction 10.9 -> 8.8; 7,000 (10x10) 8.9 -> 6.8; 15,000 (12x12) 8.9 -> 7.8, with
+// prediction 10.9 -> 10.0; beyond that one block's loads take over: 34,000 (16x16) 8.8 ->
+// 8.5 but 10.5 -> 11.3 with prediction, 58,000 (20x20) 8.9 -> 9.4.  A single frame from
+// pinned host memory, whose launches overlap the GPU's work, does not gain (20.0 -> 20.1,
+// 10x10 20.0 -> 20.5) and keeps the sum kernel.
+constexpr int kLastSumValues = 16384;
+constexpr int kLastSumGroups = 4;
+constexpr size_t kLastSumSmem = 4 * static_cast<size_t>(kLastSumGroups) * kConsumerWarps * 32;
+__host__ __device__ __forceinline__ bool last_block_sums(int S, int nact) { return S * nact <= kLastSumValues; }
+
+// Called by every consumer once the block's partials are written; ctr counts the blocks
+// of a launch and wraps.  The order of reduce_rows, four groups of 32 rows at a time.
+__device__ __forceinline__ void last_block_sum(const SumArgs& r, unsigned* ctr, float* red, int* flag, int tid) {
+    constexpr int kGroups = kLastSumGroups, kFlight = 11;
+    const int warp = tid >> 5, lane = tid & 31;
+    consumer_sync();
+    if (tid == 0) {
+        __threadfence();
+        *flag = atomicInc(ctr, gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
+    }
+    consumer_sync();
+    if (!*flag) return;
+    const bool ok = *reinterpret_cast<volatile int*>(r.status) == RTC_OK;
+    for (int base = 0; base < r.nact; base += 32 * kGroups) {
+        const int row = base + 32 * warp + lane;             // of warps 0 .. kGroups - 1: their sums
+        const bool mine = warp < kGroups && row < r.nact;
+        const float a_prev = mine ? __ldcg(r.a + row) : 0.f;
+        const float sc = mine && r.scale ? __ldg(r.scale + row) : 1.f;
+        float v[kGroups] = {0.f, 0.f, 0.f, 0.f};
+        for (int s0 = warp; s0 < r.S; s0 += kFlight * kConsumerWarps) {
+            float p[kGroups][kFlight];
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i)
+#pragma unroll
+                for (int j = 0; j < kFlight; ++j) {
+                    const int s = s0 + j * kConsumerWarps, q = base + 32 * i + lane;
+                    p[i][j] = s < r.S && q < r.nact ? __ldcg(r.partial + static_cast<size_t>(s) * r.pitch + q) : 0.f;
+                }
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i)
+#pragma unroll
+                for (int j = 0; j < kFlight; ++j)
+                    if (s0 + j * kConsumerWarps < r.S) v[i] += p[i][j];
+        }
+#pragma unroll
+        for (int i = 0; i < kGroups; ++i) red[(i * kConsumerWarps + warp) * 32 + lane] = v[i];
+        consumer_sync();
+        if (mine && ok) {
+            float t[kConsumerWarps];
+#pragma unroll
+            for (int w = 0; w < kConsumerWarps; ++w) t[w] = red[(warp * kConsumerWarps + w) * 32 + lane];
+#pragma unroll
+            for (int width = 1; width < kConsumerWarps; width <<= 1)
+#pragma unroll
+                for (int i = 0; i + width < kConsumerWarps; i += 2 * width) t[i] += t[i + width];
+            const float d = r.scale ? t[0] * sc : t[0];
+            const float an = fmaf(r.leak, a_prev, r.gain * d);
+            r.a[row] = an;
+            if (r.dm_out) r.dm_out[row] = an;
+        }
+        consumer_sync();
+    }
+}
+
 // Grid barrier over co-resident blocks: one thread per block, between two
 // block-level barriers.  The arrival is a release and the polling an acquire at
 // GPU scope, so the block's writes before the first block barrier are visible to
@@ -1178,6 +1259,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     const size_t fit = L.stage_bytes > 0 ? room / L.stage_bytes : 0;
     L.nst = static_cast<int>(fit < static_cast<size_t>(kMaxStages) ? fit : kMaxStages);
     L.smem = static_cast<size_t>(L.nst) * L.stage_bytes + extra;
+    if (!loop && last_block_sums(S, h->cfg.nact)) L.smem = std::max(L.smem, kLastSumSmem);
     L.pre_tiles = kAllTiles;
     if (!loop && min_region == 0 && h->n_valid * static_cast<long long>(h->cfg.n_wfs) <= 2ll * kConsumerWarps * L.G) {
         const bool most = 2ll * L.nst * L.stage_bytes * L.G >= h->m_bytes;
@@ -1233,3 +1315,6 @@ inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
 }
 
 }  // namespace rtc_mvm
+
+// Sum arguments of a handle (defined in mvm_stream.cu).
+rtc_mvm::SumArgs sum_args(const rtc_handle* h, float* d_dm_out);
