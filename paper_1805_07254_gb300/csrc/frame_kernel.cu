@@ -29,7 +29,7 @@
 //
 // Measured, frame after frame on one stream (one cooperative kernel with a grid barrier
 // -> this): ELT FP32 28.9 -> 23.1 us, INT8 20.9 -> 12.9, BF16 with prediction 28.4 ->
-// 25.0, six ELT sensors FP8 59.4 -> 47.4, 41x41 FP16 12.3 -> 7.9 of GPU time (9.2 with
+// 24.6, six ELT sensors FP8 59.4 -> 47.4, 41x41 FP16 12.3 -> 7.9 of GPU time (9.2 with
 // the two launches' host time, which bounds it) and 8x8 FP32 10.3 -> 6.8.  Of an FP32
 // frame the blocks stream 17 us (6.5 TB/s); slopes are known 2.9 us after the last
 // frame's sum, the hand-over to the sum takes 0.9 us and the sum 1.4.
