@@ -1198,9 +1198,12 @@ __device__ __forceinline__ void finish_host(const FrameHost& fh, const int* stat
 //   - the ring holds most of the block's share: nothing before the wait, since it fills
 //     during the pixel stage anyway (ELT INT8 13.3 us against 13.9 with one tile early
 //     and 14.1 with the whole ring; FP8 12.7, 13.2, 13.5);
-//   - it holds less than half: one tile early, the rest of the ring at the wait and two
-//     tiles more into L2, which the HBM fetches during the pixel stage (ELT FP32 23.7 us
-//     against 26.2 with the whole ring early and nothing ahead, BF16 15.9 against 17.4);
+//   - it holds less than half: one tile early, the rest of the ring at the wait and one
+//     tile more into L2, which the HBM fetches during the pixel stage (ELT FP32 23.0 us
+//     against 25.8 with the whole ring early and nothing ahead, BF16 16.5 against 17.4;
+//     a lone frame with a cold L2 31.5 and 21.4 against 33.0 and 23.0.  Two tiles ahead
+//     are 0.6 us better for BF16 frames one after another, but lone ones take 33.2 and
+//     23.0);
 //   - several pixel rounds a block (more sensors): the ring early and nothing ahead,
 //     the pixel stage itself takes the HBM (six sensors FP8 47.8 us against 50).
 using Launch = LaunchPlan;
@@ -1266,7 +1269,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     if (!loop && min_region == 0 && h->n_valid * static_cast<long long>(h->cfg.n_wfs) <= 2ll * kConsumerWarps * L.G) {
         const bool most = 2ll * L.nst * L.stage_bytes * L.G >= h->m_bytes;
         L.pre_tiles = most ? 0 : 1;
-        L.l2_ahead = most ? 0 : 2;
+        L.l2_ahead = most ? 0 : 1;
     }
     L.ok = L.nst >= 2 && L.loc_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
            S <= kMaxSlices && L.smem <= budget;
