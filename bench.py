@@ -1,15 +1,15 @@
 #!/usr/bin/env python
 """ELT-scale SCAO real-time-control benchmark on one GB300 (or N replicas).
 
-One step = one WFS frame through the whole hot path: pixel calibration +
-centre-of-gravity slopes (one kernel) then the split-K MVM fused with the
-leaky integrator (one kernel), on the 74x74-subaperture, 740x740-pixel frame
-with the 4421 x 7944 control matrix (stored FP32 by default).
+One step = one WFS frame through the whole hot path: pixel calibration,
+centre-of-gravity slopes and the partial DM vectors of the matrix slices (one
+kernel), then their sum and the leaky integrator (a second, overlapping one), on the
+74x74-subaperture, 740x740-pixel frame with the 4421 x 7944 control matrix (stored
+FP32 by default).
 
-Timing: every step is bracketed by CUDA events on the launching stream, with an
-event between the two kernels, so the same timed steps give the frame latency
-distribution (p50/p99/p99.9, RMS jitter) and the MVM kernel's duration.  L2 is
-flushed between steps by reading a 512 MiB device buffer (a read leaves only
+Timing: every step is bracketed by CUDA events on the launching stream, which gives
+the frame latency distribution (p50/p99/p99.9, RMS jitter); the two stage calls are
+timed the same way, with an event between them.  L2 is flushed between steps by reading a 512 MiB device buffer (a read leaves only
 clean lines behind, so no write-back lands inside the next step), outside the
 events.  The host
 enqueues each batch of steps behind a device-side sleep so that the GPU never
@@ -50,7 +50,7 @@ def parse_args(argv=None):
     ap.add_argument("--store", choices=["f32", "bf16", "f16", "fp8", "int8"], default="f32")
     ap.add_argument("--no-variants", action="store_true")
     ap.add_argument("--predictor", action="store_true",
-                    help="the timed controller runs the learned slope predictor (one launch per frame)")
+                    help="the timed controller runs the learned slope predictor")
     ap.add_argument("--no-loop", action="store_true")
     # the persistent-loop runs of the serving sizing: 100,000 frames each, paced at 1 kHz
     # and flat out (p99.9 over 1e5 frames rests on 100 samples)
@@ -92,11 +92,11 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-KERNEL_SOURCES = ("frame_kernel.cu", "stream_mvm.cuh", "pixel.cuh", "pred_tile.cuh")
+KERNEL_SOURCES = ("frame_kernel.cu", "mvm_stream.cu", "calib_cog.cu", "stream_mvm.cuh", "pixel.cuh", "pred_tile.cuh")
 
 
 def kernel_source_digest():
-    """sha256[:16] over the sources of the fused frame kernel."""
+    """sha256[:16] over the sources of a frame's kernels."""
     h = hashlib.sha256()
     for name in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_1805_07254_gb300", "csrc", name), "rb") as f:
@@ -500,7 +500,7 @@ def ours(args):
         variants["bf16_predictor"] = {"p50_us": round(sp["p50"], 3), "p99_us": round(sp["p99"], 3),
                                       "p999_us": round(sp["p999"], 3),
                                       "rms_jitter_us": round(sp["rms_jitter"], 3),
-                                      "kernels_per_frame": 1}
+                                      "kernels_per_frame": 3}
         rp.close()
 
     # stress sizing: six ELT WFS into one 4421 x 47664 FP8 matrix
@@ -614,13 +614,14 @@ def ours(args):
                               "mvm_stream_kernel": round(s_mvm["p50"], 3),
                               "step_two_kernels": round(s_step2["p50"], 3)},
         "stage_mvm_hbm_gbs": round(mvm_gbs, 1),
-        "roofline": {"kernel": "frame_kernel", "bound": "hbm", "achieved": round(frame_gbs, 1),
+        "roofline": {"kernel": "frame_kernel + mvm_reduce_kernel", "bound": "hbm", "achieved": round(frame_gbs, 1),
                      "peak": hbm_peak, "peak_kind": peak_kind, "unit": "GB/s",
                      "frac": round(frame_gbs / hbm_peak, 4), "traffic": traffic,
                      "algorithmic_bytes": step_bytes,
                      "launch_floor_us": round(floor_us, 3)},
         "e2e": e2e_entry(s_e2e, s_res, resident_headline, info, cfg, n_e2e, step_in_bytes, l2_bytes),
-        "gpu_launches": args.steps,
+        # (pixels and partials, sum; the predictor has a pixel stage of its own)
+        "gpu_launches": args.steps * (3 if args.predictor else 2),
         "clocks": clocks,
         "timed_wall_s_incl_flush": round(t_wall, 3),
         "variants": variants,
