@@ -413,6 +413,7 @@ cudaError_t launch_dt(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st) {
     LoopArgs a{};
     a.px = pixel_args(h, nullptr, nullptr, nullptr);
     a.mv = make_args(h, nullptr, Lc);
+    a.mv.cut = a.mv.status;             // an expired wait ends the loop: no mark for a later sum
     if (ll.l2_stream) a.mv.l2_policy = kL2Stream;
     a.frames = ll.d_frames;
     a.frame_elems = ll.frame_elems;

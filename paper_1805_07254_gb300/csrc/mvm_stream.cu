@@ -47,8 +47,9 @@ __global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g)
 }
 
 // 32 rows a block, one per lane; the order of reduce_rows (stream_mvm.cuh).  A step that
-// a bounded wait cut short (status) leaves the integrator as it was.  HOST: the last
-// block to finish writes the caller's completion record.
+// a bounded wait cut short (its own mark: record_timeout) leaves the integrator as it
+// was, and the last block to have read the mark clears it for the next step.  HOST: the
+// last block to finish writes the caller's completion record.
 template <bool HOST>
 __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, FrameHost fh) {
     __shared__ float red[kConsumerWarps * 32];
@@ -59,10 +60,10 @@ __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, Fr
     const float sc = mine && r.scale ? __ldg(r.scale + row) : 1.f;
     pdl_wait();
     float a_prev = 0.f;
-    int status = 0;
+    int cut = RTC_OK;
     if (mine) {
         a_prev = __ldcg(r.a + row);
-        status = *reinterpret_cast<volatile int*>(r.status);
+        cut = *reinterpret_cast<volatile int*>(r.cut);
     }
     // the warp's slices w, w + 14, ...: 11 in flight (152 slices are one round)
     constexpr int kFlight = 11;
@@ -82,7 +83,8 @@ __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, Fr
     }
     red[warp * 32 + lane] = v;
     __syncthreads();
-    if (mine && status == 0) {
+    if (tid == 0 && cut != RTC_OK && atomicInc(r.cutctr, gridDim.x - 1) == gridDim.x - 1) *r.cut = RTC_OK;
+    if (mine && cut == RTC_OK) {
         float t[kConsumerWarps];
 #pragma unroll
         for (int w = 0; w < kConsumerWarps; ++w) t[w] = red[w * 32 + lane];
@@ -131,8 +133,9 @@ cudaError_t configure_one() {
 
 rtc_mvm::SumArgs sum_args(const rtc_handle* h, float* d_dm_out) {
     const bool scaled = h->store == RTC_FP8_E4M3 || h->store == RTC_INT8;
-    return SumArgs{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a,  d_dm_out, h->d_status, h->sl_S,
-                   h->cfg.nact,  partial_pitch(h->cfg.nact),    h->gain, h->leak};
+    return SumArgs{h->d_partial, scaled ? h->d_scale : nullptr, h->d_a,       d_dm_out,
+                   h->d_status,  h->d_status + 1,               h->d_lastctr, h->sl_S,
+                   h->cfg.nact,  partial_pitch(h->cfg.nact),    h->gain,      h->leak};
 }
 
 cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {

@@ -248,7 +248,7 @@ int take_status(rtc_handle* h, cudaStream_t st) {
         // an aborted launch may leave the grid-barrier count short: start it afresh
         RTC_CUDA(h, cudaMemsetAsync(h->d_gridbar, 0, sizeof(unsigned long long), st));
         h->grid_epoch = 0;
-        RTC_CUDA(h, cudaMemsetAsync(h->d_status, 0, sizeof(int), st));
+        RTC_CUDA(h, cudaMemsetAsync(h->d_status, 0, 2 * sizeof(int), st));
         RTC_CUDA(h, cudaStreamSynchronize(st));
         return fail(h, code, "a bounded device wait expired (results of this step are invalid)");
     }
@@ -470,13 +470,13 @@ int rtc_create(const rtc_config* cfg, rtc_handle** out) {
         if (cudaMalloc(&h->d_a, c.nact * sizeof(float)) != cudaSuccess ||
             cudaMalloc(&h->d_partial, 2 * static_cast<size_t>(h->dev_sms) * partial_pitch(c.nact) * sizeof(float)) != cudaSuccess ||
             cudaMalloc(&h->d_frame, frame_elems * sizeof(uint16_t)) != cudaSuccess ||
-            cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess ||
+            cudaMalloc(&h->d_status, 2 * sizeof(int)) != cudaSuccess ||
             cudaMalloc(&h->d_gridbar, sizeof(unsigned long long)) != cudaSuccess ||
             cudaMalloc(&h->d_lastctr, sizeof(unsigned)) != cudaSuccess ||
             cudaMallocHost(&h->h_status, sizeof(int)) != cudaSuccess) {
             rcode = fail(nullptr, RTC_ENOMEM, "device allocation failed");
         } else if (cudaMemset(h->d_a, 0, c.nact * sizeof(float)) != cudaSuccess ||
-                   cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess ||
+                   cudaMemset(h->d_status, 0, 2 * sizeof(int)) != cudaSuccess ||
                    cudaMemset(h->d_gridbar, 0, sizeof(unsigned long long)) != cudaSuccess ||
                    cudaMemset(h->d_lastctr, 0, sizeof(unsigned)) != cudaSuccess) {
             rcode = fail(nullptr, RTC_EDEVICE, "cudaMemset failed");

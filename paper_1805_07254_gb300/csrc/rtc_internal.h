@@ -117,9 +117,11 @@ struct rtc_handle {
     float* d_partial = nullptr;     // [2][dev_sms][pitch] partial DM vectors, one per slice (scratch;
                                     // the persistent loop alternates the halves frame by frame)
     uint16_t* d_frame = nullptr;    // [n_wfs][side][side] staging for host frames
-    int* d_status = nullptr;        // device-side error word (RTC_ETIMEDOUT from bounded waits)
+    int* d_status = nullptr;        // [2] device-side error word (RTC_ETIMEDOUT from bounded waits) until
+                                    // the host takes it; mark of a per-frame launch cut short by one
     unsigned long long* d_gridbar = nullptr;  // grid-barrier arrival counter (only grows)
-    unsigned* d_lastctr = nullptr;            // finished blocks of a launch whose last block sums (wraps)
+    unsigned* d_lastctr = nullptr;            // finished blocks of a launch whose last block sums, or of
+                                              // a sum kernel that clears the mark (wraps)
     unsigned long long grid_epoch = 0;        // block arrivals expected so far on d_gridbar
 
     // persistent loop (allocated by the first rtc_run_loop)

@@ -313,7 +313,8 @@ struct Args {
     int pstride;             // nact, rounded up to the groups of 16 rows
     float* a;                // [nact] integrator state
     float gain, leak;
-    int* status;             // device error word
+    int* status;             // device error word, kept until the host reads it
+    int* cut;                // mark of this launch alone (see record_timeout)
 };
 
 struct Shared {
@@ -443,6 +444,14 @@ __device__ __forceinline__ void prefetch_rows(const Args& g, const Plan& pl, int
 // be writing shared memory when the block exits).
 __device__ __forceinline__ void rows_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// A bounded wait of this launch expired.  The error word stays set until the host reads
+// it; the mark tells the sum of this launch that partials are missing, which then leaves
+// the integrator as it was and clears the mark, so that the next frame runs as usual.
+__device__ __forceinline__ void record_timeout(const Args& g) {
+    atomicExch(g.status, RTC_ETIMEDOUT);
+    atomicExch(g.cut, RTC_ETIMEDOUT);
+}
+
 // Rows of slice tiles with rb bytes per row: R rows for the widest slice, a multiple
 // of R that still fits in a stage for narrower ones.  A row is always summed by
 // the same T lanes, so the tile height does not change any result.
@@ -492,7 +501,7 @@ __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh
         }
     }
     if (!ok && !sh.abort_flag) {
-        atomicExch(g.status, RTC_ETIMEDOUT);
+        record_timeout(g);
         sh.abort_flag = 1;
     }
     if (drain || !ok)
@@ -589,7 +598,7 @@ __device__ __forceinline__ int consume_slice(const Args& g, const Plan& pl, Shar
                                                             (tile / nst) & 1, &sh.abort_flag));
         if (!ok) {
             if (lane == 0 && !sh.abort_flag) {
-                atomicExch(g.status, RTC_ETIMEDOUT);
+                record_timeout(g);
                 sh.abort_flag = 1;
             }
             continue;     // skip the work but keep reaching the block's barriers
@@ -972,7 +981,7 @@ __device__ __forceinline__ int consume_slice_frag(const Args& g, const Plan& pl,
             if (lane == 0) mbar_arrive(smem_addr(&sh.empty_bar[st]));
         } else if (lane == 0 && !sh.abort_flag) {
             // skip the work but keep reaching the block's barriers
-            atomicExch(g.status, RTC_ETIMEDOUT);
+            record_timeout(g);
             sh.abort_flag = 1;
         }
         if (++st == nst) {
@@ -1065,7 +1074,9 @@ struct SumArgs {
     const float* scale;      // [nact] row scales, or null
     float* a;
     float* dm_out;           // [nact] or null
-    int* status;
+    int* status;             // for the caller's completion record
+    int* cut;                // set if this step's partials are incomplete (record_timeout)
+    unsigned* cutctr;        // finished blocks of a sum kernel that clears it (wraps)
     int S, nact, pitch;
     float gain, leak;
 };
@@ -1098,7 +1109,7 @@ __device__ __forceinline__ void last_block_sum(const SumArgs& r, unsigned* ctr, 
     }
     consumer_sync();
     if (!*flag) return;
-    const bool ok = *reinterpret_cast<volatile int*>(r.status) == RTC_OK;
+    const bool ok = *reinterpret_cast<volatile int*>(r.cut) == RTC_OK;
     for (int base = 0; base < r.nact; base += 32 * kGroups) {
         const int row = base + 32 * warp + lane;             // of warps 0 .. kGroups - 1: their sums
         const bool mine = warp < kGroups && row < r.nact;
@@ -1138,6 +1149,7 @@ __device__ __forceinline__ void last_block_sum(const SumArgs& r, unsigned* ctr, 
         }
         consumer_sync();
     }
+    if (tid == 0 && !ok) *r.cut = RTC_OK;        // every thread has read it
 }
 
 // Grid barrier over co-resident blocks: one thread per block, between two
@@ -1316,6 +1328,7 @@ inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
     g.gain = h->gain;
     g.leak = h->leak;
     g.status = h->d_status;
+    g.cut = h->d_status + 1;
     return g;
 }
 
