@@ -485,6 +485,9 @@ int rtc_set_predictor(rtc_handle* h, int32_t on);
  * ksplit, the number of column splits, is accepted for callers that pass one; the
  * result does not depend on it.
  *
+ * Every wait of the kernel for its own copies is bounded (200 ms).  Should one expire,
+ * the rows concerned keep their state in d_a, and their entries of d_dm_out are NaN.
+ *
  * The first call on a device configures the kernels (this may load the library's
  * device code); make that first call before any stream capture.  Calls on different
  * streams are independent (a call orders only its own buffers).

@@ -167,10 +167,12 @@ __global__ void __launch_bounds__(kThreads, 1) mvm_noalloc_kernel(NoallocArgs g)
         for (int width = 1; width < kConsumerWarps; width <<= 1)
 #pragma unroll
             for (int w = 0; w + width < kConsumerWarps; w += 2 * width) t[w] += t[w + width];
-        float d = RowScaled<DT>::v ? t[0] * g.scale[row] : t[0];
-        if (sh.abort_flag) d = __uint_as_float(0x7fc00000u);  // a copy that never landed: not a number
-        const float an = fmaf(g.leak, g.a[row], g.gain * d);
-        g.a[row] = an;
+        const float d = RowScaled<DT>::v ? t[0] * g.scale[row] : t[0];
+        float an = fmaf(g.leak, g.a[row], g.gain * d);
+        // a copy that never landed: the command is not a number, the state stays as it
+        // was, so that the next call starts from it
+        if (sh.abort_flag) an = __uint_as_float(0x7fc00000u);
+        else g.a[row] = an;
         if (g.dm_out) g.dm_out[row] = an;
     }
 }
