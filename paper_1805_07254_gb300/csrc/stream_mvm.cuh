@@ -467,7 +467,9 @@ __device__ __forceinline__ int tile_rows(const Args& g, int rb) {
 // in flight).  The ring fills before the block's slopes are known and then waits for
 // its consumers.  A per-frame kernel requests its first pre_tiles tiles before its
 // predecessor is complete, the others after (the persistent loop has no predecessor),
-// and l2_ahead further ones into L2 (see Launch::pre_tiles).
+// and l2_ahead further ones into L2 (see Launch::pre_tiles).  pre_tiles is at most the
+// ring's stages: the bounded wait for a stage starts after the unbounded one for the
+// predecessor, whose run time is not this kernel's.
 __device__ __forceinline__ int produce(const Args& g, const Plan& pl, Shared& sh, int tl0 = 0, bool drain = true) {
     int tl = tl0;
     bool ok = true;
@@ -1218,8 +1220,9 @@ __device__ __forceinline__ void finish_host(const FrameHost& fh, const int* stat
 //     23.0);
 //   - several pixel rounds a block (more sensors): the ring early and nothing ahead,
 //     the pixel stage itself takes the HBM (six sensors FP8 47.8 us against 50).
+//     Prediction frames too, whose blocks have the whole pixel kernel to wait for.
 using Launch = LaunchPlan;
-constexpr int kAllTiles = 1 << 30;
+constexpr int kNoPredecessor = -1;
 
 // min_region: shared-memory scratch a fused phase needs.  loop: the persistent kernel,
 // which also sums its rows (integrator state, row scales and warp sums in shared
@@ -1277,7 +1280,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     L.nst = static_cast<int>(fit < static_cast<size_t>(kMaxStages) ? fit : kMaxStages);
     L.smem = static_cast<size_t>(L.nst) * L.stage_bytes + extra;
     if (!loop && last_block_sums(S, h->cfg.nact)) L.smem = std::max(L.smem, kLastSumSmem);
-    L.pre_tiles = kAllTiles;
+    L.pre_tiles = loop ? kNoPredecessor : L.nst;
     if (!loop && min_region == 0 && h->n_valid * static_cast<long long>(h->cfg.n_wfs) <= 2ll * kConsumerWarps * L.G) {
         const bool most = 2ll * L.nst * L.stage_bytes * L.G >= h->m_bytes;
         L.pre_tiles = most ? 0 : 1;
