@@ -680,7 +680,8 @@ __device__ __forceinline__ int consume_slice(const Args& g, const Plan& pl, Shar
 //     (What falls below FP16's subnormals, 2^-61 of the largest slope in the third
 //     part, is dropped.)
 // Products are exact and accumulate in FP32, and the three column sums meet at the end.
-// Infinite and NaN slopes go whole into the first part.  Against 64 bits the commands
+// Infinite and NaN slopes go whole into the first part, and an infinite sum of first
+// parts (an infinite slope or matrix entry) is the row's sum.  Against 64 bits the commands
 // are as near as the FP32 chains' were or nearer (relative 2-norm: ELT FP16 41x41 1.2e-7
 // against 1.3e-7, six sensors FP8 2.3e-7 against 2.5e-7, BF16 loop 1.7e-7 against 2.1e-7).
 // Measured, frame after frame, with FP32 chains -> so: ELT INT8 17.0 -> 13.7 us, six
@@ -929,6 +930,9 @@ __device__ __forceinline__ void frag_dot(uint32_t at, uint32_t gap, int K, int l
             const float p2 = __shfl_xor_sync(0xffffffffu, acc[i][2 * r], 1);
             v[i][r] = HalfKind<DT>::v ? fmaf(fmaf(p2, 0x1p-11f, acc[i][2 * r + 1]), 0x1p-11f, acc[i][2 * r])
                                       : acc[i][2 * r] + (acc[i][2 * r + 1] + p2);
+            // an infinite matrix entry (2-byte stores): the second and third parts may be zero, and
+            // infinity times zero is no part of the sum
+            if (ES == 2 && isinf(acc[i][2 * r])) v[i][r] = acc[i][2 * r];
         }
 }
 
