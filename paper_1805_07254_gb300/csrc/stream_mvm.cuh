@@ -677,8 +677,10 @@ __device__ __forceinline__ int consume_slice(const Args& g, const Plan& pl, Shar
 //     splits: nothing overflows, and the range is FP32's own);
 //   - FP16: 11 bits, 11 and 2, the second and third scaled by 2^11 and 2^22, after a
 //     power of two per slice that brings the slice's largest slope just below 2^15.
-//     (What falls below FP16's subnormals, 2^-61 of the largest slope in the third
-//     part, is dropped.)
+// The split loses bits of slopes below 2^-37 of the slice's largest (FP16), where FP16's
+// subnormals end, or below 2^-102 (BF16).  A slice that holds such a slope is marked and
+// its rows are summed once more as FP32 chains (wide_slices): a matrix may well be zero
+// where a dead subaperture's slope is huge.
 // Products are exact and accumulate in FP32, and the three column sums meet at the end.
 // Infinite and NaN slopes go whole into the first part, and an infinite sum of first
 // parts (an infinite slope or matrix entry) is the row's sum.  Against 64 bits the commands
@@ -753,8 +755,9 @@ __device__ __forceinline__ void slope_scale(const float* sv, int K, int lane, fl
 
 // The parts of column c of a slice of K columns into its B fragments: the step, quarter
 // t and place j of the matrix elements the lanes hold (slice_elem_offset's column order).
+// scale: set to 0 where the parts do not hold all of v.
 template <int DT>
-__device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, float up) {
+__device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, float up, float* scale) {
     const bool finite = (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
     const int k32 = Esize<DT>::v == 1 ? K & ~31 : 0, rest = c - (K & ~15);
     int step = c >> 4, t = (c & 15) >> 2, j = c & 3;
@@ -768,6 +771,7 @@ __device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, fl
     }
     unsigned short* out = reinterpret_cast<unsigned short*>(frag) + step * 48 + t * 4 + j;
     float r = HalfKind<DT>::v ? v * up : v;
+    if (v != 0.f && fabsf(r) < (HalfKind<DT>::v ? 0x1p-23f : 0x1p-102f)) *scale = 0.f;
 #pragma unroll
     for (int n = 0; n < 3; ++n) {
         unsigned short d;
@@ -808,7 +812,8 @@ __device__ __forceinline__ void make_bfrag(const Args& g, const Plan& pl, int ti
         }
         if (one) consumer_sync();
         else __syncwarp();
-        for (int c = one ? tid : lane; c < K; c += one ? kConsumers : 32) put_parts<DT>(frag, K, c, sv[c], up);
+        for (int c = one ? tid : lane; c < K; c += one ? kConsumers : 32)
+            put_parts<DT>(frag, K, c, sv[c], up, pl.bscale + (s - pl.sb0));
     }
 }
 
@@ -939,10 +944,11 @@ __device__ __forceinline__ void frag_dot(uint32_t at, uint32_t gap, int K, int l
 // The tiles of one slice in fragment order; returns the running tile count.  A warp
 // takes the groups of 16 rows w, w + 14, ... of a tile, up to four at a time.  Each row's
 // sum depends on the slice alone.  (The padding rows of the last group have their
-// place in the partial vectors too: no row is tested.)
+// place in the partial vectors too: no row is tested.)  wide: set if the slice is marked
+// (its sums come out as zeros and are replaced later).
 template <int DT, bool SMALL>
 __device__ __forceinline__ int consume_slice_frag(const Args& g, const Plan& pl, Shared& sh, int tid, int tile, int s,
-                                                  int rb, int lo) {
+                                                  int rb, int lo, bool& wide) {
     const int nact = g.nact, nst = g.nst, stage_bytes = g.stage_bytes;
     const int warp = tid >> 5, lane = tid & 31;
     const int K = rb / Esize<DT>::v;
@@ -955,6 +961,7 @@ __device__ __forceinline__ int consume_slice_frag(const Args& g, const Plan& pl,
         if (K & 15) sb.last = bfrag(frag, K >> 4, lane);
     }
     const float down = pl.bscale[s - pl.sb0];
+    wide |= down == 0.f;
     const bool first = (lane & 3) == 0;
     float* out = g.partial + static_cast<size_t>(s) * g.pstride + warp * 16 + (lane >> 2);
     const int tr = tile_rows(g, rb);
@@ -998,6 +1005,40 @@ __device__ __forceinline__ int consume_slice_frag(const Args& g, const Plan& pl,
     return tile;
 }
 
+// A stored entry as FP32 (INT8 codes are stored flipped).
+template <int DT>
+__device__ __forceinline__ float stored_value(const unsigned char* p) {
+    if constexpr (Esize<DT>::v == 2) {
+        const unsigned short u = __ldg(reinterpret_cast<const unsigned short*>(p));
+        return DT == RTC_BF16 ? __uint_as_float(static_cast<uint32_t>(u) << 16) : __half2float(__ushort_as_half(u));
+    } else {
+        const unsigned char u = __ldg(p);
+        return DT == RTC_INT8 ? static_cast<float>(static_cast<int>(u) - 128) : e4m3x2_to_float2(u).x;
+    }
+}
+
+// The rows of the block's marked slices as FP32 chains, from global memory: for a case too
+// rare to hold registers or code in the loops above, and as near as the other sums.
+template <int DT>
+__device__ __forceinline__ void wide_slices(const Args& g, const Plan& pl, int tid) {
+    constexpr int ES = Esize<DT>::v;
+    consumer_sync();                                         // the sums that these replace are out
+    for (int s = pl.sb0; s < pl.sb1; ++s) {
+        if (pl.bscale[s - pl.sb0] != 0.f) continue;
+        const int rb = __ldg(g.sl.rowbytes + s);
+        const long long off = __ldg(g.sl.off + s);
+        const float* sv = pl.loc + (__ldg(g.sl.loc + s) - pl.loc0);
+        float* out = g.partial + static_cast<size_t>(s) * g.pstride;
+        for (int row = tid; row < g.nact; row += kConsumers) {
+            float acc = 0.f;
+#pragma unroll 4
+            for (int c = 0; c < rb / ES; ++c)
+                acc = fmaf(stored_value<DT>(g.M + slice_elem_offset(off, rb, row, c * ES, ES)), sv[c], acc);
+            out[row] = acc;
+        }
+    }
+}
+
 // The consumer warps, after a consumer barrier that completes the block's slopes: every
 // tile of the block's slices, one partial vector per
 // slice (partial[s][row] = the row's dot product with the slice's slopes, in unit
@@ -1011,6 +1052,7 @@ __device__ __forceinline__ int consume(const Args& g, const Plan& pl, Shared& sh
         make_bfrag<DT>(g, pl, tid);
         consumer_sync();
     }
+    bool wide = false;                                       // the same on every thread
     for (int s = pl.sb0; s < pl.sb1; ++s) {
         int rb_next = 0, lo_next = 0;
         if (s + 1 < pl.sb1) {
@@ -1023,12 +1065,14 @@ __device__ __forceinline__ int consume(const Args& g, const Plan& pl, Shared& sh
             else if (u == 8) tile = consume_slice<DT, 8>(g, pl, sh, tid, tile, s, rb, lo);
             else tile = consume_slice<DT, 4>(g, pl, sh, tid, tile, s, rb, lo);
         } else {
-            tile = rb <= 64 * Esize<DT>::v ? consume_slice_frag<DT, true>(g, pl, sh, tid, tile, s, rb, lo)
-                                           : consume_slice_frag<DT, false>(g, pl, sh, tid, tile, s, rb, lo);
+            tile = rb <= 64 * Esize<DT>::v ? consume_slice_frag<DT, true>(g, pl, sh, tid, tile, s, rb, lo, wide)
+                                           : consume_slice_frag<DT, false>(g, pl, sh, tid, tile, s, rb, lo, wide);
         }
         rb = rb_next;
         lo = lo_next;
     }
+    if constexpr (DT != RTC_F32)
+        if (wide) wide_slices<DT>(g, pl, tid);
     return tile;
 }
 
