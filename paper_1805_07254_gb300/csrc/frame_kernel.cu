@@ -78,7 +78,8 @@ __device__ __forceinline__ void pixel_stage(const rtc_pixel::PixelArgs& px, cons
 }
 
 // LAST: the last block also sums (last_block_sum), and the launch is the whole frame.
-template <int DT, int NPX, bool HOST, bool LAST>
+// CHAIN: small slices (chain_rule).
+template <int DT, int NPX, bool HOST, bool LAST, bool CHAIN>
 __global__ void __launch_bounds__(kFrameRegThreads, 1)
 frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -101,7 +102,7 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     pixel_stage<NPX, HOST, true>(px, g, pl, fh, slot, pos0, tid);
     pdl_wait();                         // before the partials of the last frame are overwritten
     consumer_sync();
-    consume<DT>(g, pl, sh, tid, 0);
+    consume<DT, CHAIN>(g, pl, sh, tid, 0);
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kThreads, 1) frame_slopes_kernel(rtc_pixel::Pi
 // the kernel before this one.  That kernel lets this one start at once, so that the ring
 // fills and the network's weights arrive while the pixel stage waits for the frame; the
 // history is read after the wait.
-template <int DT, bool LAST>
+template <int DT, bool LAST, bool CHAIN>
 __global__ void __launch_bounds__(kFrameRegThreads, 1)
 frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned* ctr) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -153,21 +154,29 @@ frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned*
             pl.loc[axis ? iy : ix] = v;
         });
     consumer_sync();
-    consume<DT>(g, pl, sh, tid, 0);
+    consume<DT, CHAIN>(g, pl, sh, tid, 0);
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
     }
 }
 
-template <int DT, int NPX>
-cudaError_t launch_npx(const rtc_handle* h, const Launch& L, const rtc_pixel::PixelArgs& px, const Args& g,
+template <int DT, int NPX, bool CHAIN>
+cudaError_t launch_chain(const rtc_handle* h, const Launch& L, const rtc_pixel::PixelArgs& px, const Args& g,
                        const FrameHost* fh, bool last, const SumArgs& sa, cudaStream_t st) {
     const dim3 grid(L.G), block(kThreads);
     unsigned* ctr = h->d_lastctr;
-    if (fh) return launch_pdl(frame_kernel<DT, NPX, true, false>, grid, block, L.smem, st, px, g, *fh, sa, ctr);
-    if (last) return launch_pdl(frame_kernel<DT, NPX, false, true>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
-    return launch_pdl(frame_kernel<DT, NPX, false, false>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
+    if (fh) return launch_pdl(frame_kernel<DT, NPX, true, false, CHAIN>, grid, block, L.smem, st, px, g, *fh, sa, ctr);
+    if (last)
+        return launch_pdl(frame_kernel<DT, NPX, false, true, CHAIN>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
+    return launch_pdl(frame_kernel<DT, NPX, false, false, CHAIN>, grid, block, L.smem, st, px, g, FrameHost{}, sa, ctr);
+}
+
+template <int DT, int NPX>
+cudaError_t launch_npx(const rtc_handle* h, const Launch& L, const rtc_pixel::PixelArgs& px, const Args& g,
+                       const FrameHost* fh, bool last, const SumArgs& sa, cudaStream_t st) {
+    return L.chain ? launch_chain<DT, NPX, CanChain<DT>::v>(h, L, px, g, fh, last, sa, st)
+                   : launch_chain<DT, NPX, false>(h, L, px, g, fh, last, sa, st);
 }
 
 template <int DT>
@@ -201,7 +210,9 @@ cudaError_t launch_dt(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, f
         if (!fh) e = launch_calib_cog(h, d_frame, d_s_meas, d_s2, true, st);
         else if (n10) e = launch_pdl(frame_slopes_kernel<10>, grid, block, 0, st, px, g, *fh);
         else e = launch_pdl(frame_slopes_kernel<0>, grid, block, 0, st, px, g, *fh);
-        const auto k = last ? frame_pred_kernel<DT, true> : frame_pred_kernel<DT, false>;
+        constexpr bool kCan = CanChain<DT>::v;
+        const auto k = L.chain ? (last ? frame_pred_kernel<DT, true, kCan> : frame_pred_kernel<DT, false, kCan>)
+                               : (last ? frame_pred_kernel<DT, true, false> : frame_pred_kernel<DT, false, false>);
         if (e == cudaSuccess) e = launch_pdl(k, grid, block, L.smem, st, g, pred_args(h), head, sa, h->d_lastctr);
     }
     return e == cudaSuccess && !last ? launch_sum(h, d_dm_out, st, fh) : e;
@@ -212,21 +223,27 @@ cudaError_t configure(K kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kDynSmemBudget));
 }
 
-template <int DT, int NPX>
+template <int DT, int NPX, bool CHAIN>
 cudaError_t configure_npx() {
-    cudaError_t e = configure(frame_kernel<DT, NPX, false, false>);
-    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, false, true>);
-    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, true, false>);
+    cudaError_t e = configure(frame_kernel<DT, NPX, false, false, CHAIN>);
+    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, false, true, CHAIN>);
+    if (e == cudaSuccess) e = configure(frame_kernel<DT, NPX, true, false, CHAIN>);
+    return e;
+}
+
+template <int DT, bool CHAIN>
+cudaError_t configure_chain() {
+    cudaError_t e = configure_npx<DT, 10, CHAIN>();
+    if (e == cudaSuccess) e = configure_npx<DT, 0, CHAIN>();
+    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, false, CHAIN>);
+    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, true, CHAIN>);
     return e;
 }
 
 template <int DT>
 cudaError_t configure_dt() {
-    cudaError_t e = configure_npx<DT, 10>();
-    if (e == cudaSuccess) e = configure_npx<DT, 0>();
-    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, false>);
-    if (e == cudaSuccess) e = configure(frame_pred_kernel<DT, true>);
-    return e;
+    const cudaError_t e = configure_chain<DT, false>();
+    return e == cudaSuccess && CanChain<DT>::v ? configure_chain<DT, CanChain<DT>::v>() : e;
 }
 
 }  // namespace

@@ -148,7 +148,7 @@ __device__ __forceinline__ void st_release_sys(unsigned long long* p, unsigned l
     asm volatile("st.release.sys.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-template <int DT, int NPX, bool PRED>
+template <int DT, int NPX, bool PRED, bool CHAIN>
 __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
         Args mv = L.mv;
         mv.partial = L.mv.partial + (k & 1) * L.partial_stride;
         RTC_LOOP_STAMP(2);
-        tile = consume<DT>(mv, pl, sh, tid, tile);
+        tile = consume<DT, CHAIN>(mv, pl, sh, tid, tile);
         RTC_LOOP_STAMP(3);
         consumer_sync();
         if (tid == 0) grid_barrier(L.gridbar, G * (kBarriers * k + kBarriers), L.mv.status, &sh.abort_flag);
@@ -364,8 +364,9 @@ __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
 template <int DT, int NPX, bool PRED>
 cudaError_t launch_t(const Launch& Lc, LoopArgs a, cudaStream_t st) {
     void* args[] = {&a};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(loop_kernel<DT, NPX, PRED>),
-                                       dim3(Lc.G), dim3(kThreads), args, Lc.smem, st);
+    const auto k = Lc.chain ? loop_kernel<DT, NPX, PRED, CanChain<DT>::v> : loop_kernel<DT, NPX, PRED, false>;
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k), dim3(Lc.G), dim3(kThreads), args, Lc.smem,
+                                       st);
 }
 
 }  // namespace
@@ -453,8 +454,12 @@ cudaError_t launch_dt(rtc_handle* h, const LoopLaunch& ll, cudaStream_t st) {
 
 template <int DT, int NPX, bool PRED>
 cudaError_t configure_t() {
-    return cudaFuncSetAttribute(loop_kernel<DT, NPX, PRED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kDynSmemBudget));
+    const int bytes = static_cast<int>(kDynSmemBudget);
+    const cudaError_t e =
+        cudaFuncSetAttribute(loop_kernel<DT, NPX, PRED, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess || !CanChain<DT>::v) return e;
+    return cudaFuncSetAttribute(loop_kernel<DT, NPX, PRED, CanChain<DT>::v>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 template <int DT>

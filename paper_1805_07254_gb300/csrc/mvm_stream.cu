@@ -25,7 +25,7 @@ namespace {
 
 using namespace rtc_mvm;
 
-template <int DT>
+template <int DT, bool CHAIN>
 __global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kFrameRegThreads, 1) mvm_stream_kernel(Args g)
     pdl_wait();
     gather_local(g, pl, tid, g.s, true);
     consumer_sync();
-    consume<DT>(g, pl, sh, tid, 0);
+    consume<DT, CHAIN>(g, pl, sh, tid, 0);
 }
 
 // 32 rows a block, one per lane; the order of reduce_rows (stream_mvm.cuh).  A step that
@@ -119,14 +119,19 @@ cudaError_t launch_stream(rtc_handle* h, const float* d_s, float* d_dm_out, cuda
     const Launch& L = frame_plan(h, rtc_pred::kSmemBytes, false);
     if (!L.ok) return cudaErrorInvalidValue;
     const Args g = make_args(h, d_s, L);
-    const cudaError_t e = launch_pdl(mvm_stream_kernel<DT>, dim3(L.G), dim3(kThreads), L.smem, st, g);
+    const auto k = L.chain ? mvm_stream_kernel<DT, CanChain<DT>::v> : mvm_stream_kernel<DT, false>;
+    const cudaError_t e = launch_pdl(k, dim3(L.G), dim3(kThreads), L.smem, st, g);
     return e == cudaSuccess ? launch_sum(h, d_dm_out, st) : e;
 }
 
 template <int DT>
 cudaError_t configure_one() {
-    return cudaFuncSetAttribute(mvm_stream_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kDynSmemBudget));
+    const int bytes = static_cast<int>(kDynSmemBudget);
+    const cudaError_t e =
+        cudaFuncSetAttribute(mvm_stream_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess || !CanChain<DT>::v) return e;
+    return cudaFuncSetAttribute(mvm_stream_kernel<DT, CanChain<DT>::v>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                bytes);
 }
 
 }  // namespace

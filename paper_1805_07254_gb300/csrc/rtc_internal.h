@@ -65,7 +65,7 @@ inline int partial_pitch(int nact) { return (nact + 15) / 16 * 16; }
 struct LaunchPlan {
     int G, T, R, nst, stage_bytes, loc_floats, row_floats, max_slices, bf_floats, pre_tiles, l2_ahead;
     size_t smem, region;
-    bool ok;
+    bool chain, ok;
 };
 
 struct rtc_handle {

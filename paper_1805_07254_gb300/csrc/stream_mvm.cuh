@@ -145,6 +145,11 @@ __device__ __forceinline__ uint32_t lds32(uint32_t addr) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
 }
+__device__ __forceinline__ uint32_t lds16(uint32_t addr) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+    return v;
+}
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
     uint2 v;
     asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
@@ -755,9 +760,9 @@ __device__ __forceinline__ void slope_scale(const float* sv, int K, int lane, fl
 
 // The parts of column c of a slice of K columns into its B fragments: the step, quarter
 // t and place j of the matrix elements the lanes hold (slice_elem_offset's column order).
-// scale: set to 0 where the parts do not hold all of v.
+// Returns whether they may not hold all of v.
 template <int DT>
-__device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, float up, float* scale) {
+__device__ __forceinline__ bool put_parts(float* frag, int K, int c, float v, float up) {
     const bool finite = (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u;
     const int k32 = Esize<DT>::v == 1 ? K & ~31 : 0, rest = c - (K & ~15);
     int step = c >> 4, t = (c & 15) >> 2, j = c & 3;
@@ -771,7 +776,7 @@ __device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, fl
     }
     unsigned short* out = reinterpret_cast<unsigned short*>(frag) + step * 48 + t * 4 + j;
     float r = HalfKind<DT>::v ? v * up : v;
-    if (v != 0.f && fabsf(r) < (HalfKind<DT>::v ? 0x1p-23f : 0x1p-102f)) *scale = 0.f;
+    const bool lost = v != 0.f && fabsf(r) < (HalfKind<DT>::v ? 0x1p-23f : 0x1p-102f);
 #pragma unroll
     for (int n = 0; n < 3; ++n) {
         unsigned short d;
@@ -787,6 +792,7 @@ __device__ __forceinline__ void put_parts(float* frag, int K, int c, float v, fl
         }
         out[n * 16] = d;
     }
+    return lost;
 }
 
 // B fragments of the block's slices from its local slopes, and what each slice's sums
@@ -812,8 +818,9 @@ __device__ __forceinline__ void make_bfrag(const Args& g, const Plan& pl, int ti
         }
         if (one) consumer_sync();
         else __syncwarp();
-        for (int c = one ? tid : lane; c < K; c += one ? kConsumers : 32)
-            put_parts<DT>(frag, K, c, sv[c], up, pl.bscale + (s - pl.sb0));
+        bool lost = false;
+        for (int c = one ? tid : lane; c < K; c += one ? kConsumers : 32) lost |= put_parts<DT>(frag, K, c, sv[c], up);
+        if (lost) pl.bscale[s - pl.sb0] = 0.f;               // the mark of a slice for wide_slices
     }
 }
 
@@ -1039,13 +1046,92 @@ __device__ __forceinline__ void wide_slices(const Args& g, const Plan& pl, int t
     }
 }
 
+// One row of a fragment-order slice of K columns on the CUDA cores: row r of the group of
+// 16 rows at shared address at, its terms added in column order.
+template <int DT>
+__device__ __forceinline__ float chain_row(uint32_t at, int K, int r, const float* sv) {
+    constexpr int ES = Esize<DT>::v;
+    const int g8 = r & 7, half = r >> 3;
+    // <a 4-byte word, or its lower half, its slopes>; INT8 codes are stored flipped
+    auto word = [](float acc, uint32_t w, const float* s) {
+        return word_dot<DT>(acc, DT == RTC_INT8 ? w ^ 0x80808080u : w, s);
+    };
+    auto pair = [&](float acc, uint32_t a, const float* s) {
+        if constexpr (ES == 2) return word(acc, lds32(a), s);
+        else {
+            const uint32_t w = lds16(a);
+            const float2 p = DT == RTC_INT8 ? make_float2(i8_to_float(w, 0), i8_to_float(w, 1)) : e4m3x2_to_float2(w);
+            return fmaf(p.y, s[1], fmaf(p.x, s[0], acc));
+        }
+    };
+    float acc = 0.f;
+    int c = 0;
+    if constexpr (ES == 1)
+        for (; c + 32 <= K; c += 32, at += 512)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const uint2 w = lds64(at + ((g8 * 4 + t) * 2 + half) * 8);
+                acc = word(word(acc, w.x, sv + c + 8 * t), w.y, sv + c + 8 * t + 4);
+            }
+    for (; c + 16 <= K; c += 16, at += 256 * ES)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t a = at + ((g8 * 4 + t) * 2 + half) * 4 * ES;
+            if constexpr (ES == 1) {
+                acc = word(acc, lds32(a), sv + c + 4 * t);
+            } else {
+                const uint2 w = lds64(a);
+                acc = word(word(acc, w.x, sv + c + 4 * t), w.y, sv + c + 4 * t + 2);
+            }
+        }
+    if (c + 8 <= K) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) acc = pair(acc, at + ((g8 * 4 + t) * 2 + half) * 2 * ES, sv + c + 2 * t);
+        at += 128 * ES;
+        c += 8;
+    }
+    const int pairs = (K - c) >> 1;
+    for (int t = 0; t < pairs; ++t) acc = pair(acc, at + ((g8 * pairs + t) * 2 + half) * 2 * ES, sv + c + 2 * t);
+    return acc;
+}
+
+// The block's slices in fragment order by FP32 chains, a row a thread, each row's terms in
+// column order; returns the running tile count.
+template <int DT>
+__device__ __forceinline__ int consume_chain(const Args& g, const Plan& pl, Shared& sh, int tid, int tile) {
+    const int lane = tid & 31;
+    for (int s = pl.sb0; s < pl.sb1; ++s) {
+        const int rb = s == pl.sb0 ? pl.rb0 : __ldg(g.sl.rowbytes + s);
+        const float* sv = pl.loc + (s == pl.sb0 ? 0 : __ldg(g.sl.loc + s) - pl.loc0);
+        const int K = rb / Esize<DT>::v, tr = tile_rows(g, rb);
+        float* out = g.partial + static_cast<size_t>(s) * g.pstride;
+        for (int row0 = 0; row0 < g.nact; row0 += tr, ++tile) {
+            const int st = tile % g.nst;
+            if (__all_sync(0xffffffffu, wait_phase(smem_addr(&sh.full_bar[st]), (tile / g.nst) & 1, &sh.abort_flag))) {
+                const uint32_t stage = pl.ring + st * g.stage_bytes;
+                const int rows = min(tr, g.nact - row0);
+                for (int r = tid; r < rows; r += kConsumers)
+                    out[row0 + r] = chain_row<DT>(stage + (r >> 4) * 16 * rb, K, r & 15, sv);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_addr(&sh.empty_bar[st]));
+            } else if (lane == 0 && !sh.abort_flag) {
+                record_timeout(g);
+                sh.abort_flag = 1;
+            }
+        }
+    }
+    return tile;
+}
+
 // The consumer warps, after a consumer barrier that completes the block's slopes: every
 // tile of the block's slices, one partial vector per
 // slice (partial[s][row] = the row's dot product with the slice's slopes, in unit
 // order).  tile0: the running tile count at entry; returns the count at exit.  The
-// next slice's layout is fetched while the present one is consumed.
-template <int DT>
+// next slice's layout is fetched while the present one is consumed.  CHAIN: see
+// chain_rule.
+template <int DT, bool CHAIN>
 __device__ __forceinline__ int consume(const Args& g, const Plan& pl, Shared& sh, int tid, int tile0) {
+    if constexpr (CHAIN) return consume_chain<DT>(g, pl, sh, tid, tile0);
     int tile = tile0;
     int rb = pl.rb0, lo = 0;
     if constexpr (DT != RTC_F32) {
@@ -1270,6 +1356,19 @@ __device__ __forceinline__ void finish_host(const FrameHost& fh, const int* stat
 //     the pixel stage itself takes the HBM (six sensors FP8 47.8 us against 50).
 //     Prediction frames too, whose blocks have the whole pixel kernel to wait for.
 using Launch = LaunchPlan;
+
+// Small slices of 1- and 2-byte stores: FP32 chains instead of the tensor cores.  Splitting
+// the slopes, the two barriers around it and the fragments take 0.6 us whatever the size,
+// and a thread's share of a small slice, its columns times the rows it takes, is less.
+// Measured, loop (host to host) and frame after frame, INT8, tensor cores -> chains:
+// 8x8 12.6 -> 11.4 and 6.5 -> 5.6 us, 26x26 (8 columns x 2 rows) 12.8 -> 12.4 and 6.1 ->
+// 5.4, 34x34 (12 x 3) 13.1 -> 12.7 and 6.4 -> 6.0; beyond the line FP16 41x41 (18 x 4)
+// 13.7 -> 14.0 and 6.9 -> 7.4.  Every slice of a matrix goes the same way, in all kernels.
+constexpr int kChainSteps = 40;
+template <int DT> struct CanChain { static constexpr bool v = DT != RTC_F32; };
+inline bool chain_rule(int max_rb, int esz, int nact) {
+    return esz < 4 && max_rb / esz * static_cast<long long>((nact + kConsumers - 1) / kConsumers) <= kChainSteps;
+}
 constexpr int kNoPredecessor = -1;
 
 // min_region: shared-memory scratch a fused phase needs.  loop: the persistent kernel,
@@ -1295,6 +1394,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     L.loc_floats = (max_loc + 3) / 4 * 4;
     L.row_floats = (h->cfg.nact + L.G - 1) / L.G;
     L.region = (min_region + 15) / 16 * 16;
+    L.chain = chain_rule(max_rb, esz, h->cfg.nact);
     L.bf_floats = frag ? bfrag_floats(L.loc_floats) : 0;
     const size_t slopes = 4 * static_cast<size_t>(L.loc_floats + L.bf_floats + (frag ? L.max_slices : 0));
     size_t extra = L.region + slopes + 8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
