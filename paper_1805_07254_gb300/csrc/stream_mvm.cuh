@@ -172,6 +172,15 @@ __host__ __device__ __forceinline__ int row_unit(int rb) {
     if (rb % 4 == 0 && (rb / 4) % 2 == 1) return 4;
     return 0;
 }
+// Bytes of a slice's row of 2 n entries until an access unit exists, and the floats of its
+// slopes.  (Fragment-order slices are neither padded so, nor their slopes; the limit on
+// a block's slopes counts every store alike.)
+inline int row_bytes(int n, int esz) {
+    int rb = (2 * n * esz + 3) / 4 * 4;
+    while (row_unit(rb) == 0) rb += 4;
+    return rb;
+}
+inline int slope_floats(int n, int esz) { return (row_bytes(n, esz) / esz + 3) / 4 * 4; }
 // A handle's INT8 codes are stored with the sign bit flipped (code + 128 as an unsigned
 // byte), which widen4 wants.
 constexpr unsigned char kInt8Flip = 0x80;
@@ -1388,7 +1397,12 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
         const int s0 = static_cast<int>(static_cast<long long>(S) * b / L.G);
         const int s1 = static_cast<int>(static_cast<long long>(S) * (b + 1) / L.G);
         max_loc = std::max(max_loc, h->sl_loc[s1] - h->sl_loc[s0]);
-        for (int s = s0; s < s1; ++s) max_rb = std::max(max_rb, h->sl_rowbytes[s]);
+        int floats = 0;
+        for (int s = s0; s < s1; ++s) {
+            max_rb = std::max(max_rb, h->sl_rowbytes[s]);
+            floats += slope_floats(h->sl_g0[s + 1] - h->sl_g0[s], esz);
+        }
+        max_floats = std::max(max_floats, floats);
         L.max_slices = std::max(L.max_slices, s1 - s0);
     }
     L.loc_floats = (max_loc + 3) / 4 * 4;
