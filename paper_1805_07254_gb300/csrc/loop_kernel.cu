@@ -349,12 +349,13 @@ __global__ void __launch_bounds__(kThreads, 1) loop_kernel(LoopArgs L) {
             __threadfence_system();
             const unsigned long long prev = atomicAdd(L.donectr, 1ull);
             if (prev + 1 == G * (k + 1)) {
+                const unsigned long long t_done = global_ns();   // the commands are out: no fence in it
                 __threadfence();          // the fences over the host link: see finish_host
                 rtc_loop_done* d = L.done + slot;
                 // the latest time a block had its rows; cleared for frame k + 2, whose
                 // blocks start after the grid barrier of frame k + 1
                 d->t_seen = atomicExch(L.t_seen + (k & 1), 0ull);
-                d->t_done = global_ns();
+                d->t_done = t_done;
                 st_release_sys(&d->seq, k + 1);
             }
         }
