@@ -125,15 +125,13 @@ void cut_slices(rtc_handle* h, const std::vector<int>& g0, int esz, std::vector<
     int loc = 0;
     for (int s = 0; s < S; ++s) {
         const int n = g0[s + 1] - g0[s];
-        int rb = 2 * n * esz;
-        if (!h->sl_frag)
-            while (rtc_mvm::row_unit(rb) == 0) rb += 4;   // a bank-conflict-free access unit
+        const int rb = h->sl_frag ? 2 * n * esz : rtc_mvm::row_bytes(n, esz);
         const long long rows = h->sl_frag ? (nact + 15) / 16 * 16ll : nact;
         h->sl_off[s] = off;
         h->sl_rowbytes[s] = rb;
         off += (rows * rb + 15) / 16 * 16;
         h->sl_loc[s] = loc;
-        loc += h->sl_frag ? (2 * n + 15) / 16 * 16 : (rb / esz + 3) / 4 * 4;
+        loc += h->sl_frag ? (2 * n + 15) / 16 * 16 : rtc_mvm::slope_floats(n, esz);
     }
     h->sl_loc[S] = loc;
     h->m_bytes = off;

@@ -62,7 +62,7 @@ constexpr int kMaxRowsPerThread = 32;
 // Largest matrix streamed with the default L2 policy (of the 126 MB L2).
 constexpr long long kL2KeepBytes = 80ll << 20;
 constexpr unsigned long long kWaitNs = 200ull * 1000 * 1000;
-constexpr int kMaxLocalFloats = 8192;              // slopes of a block's slices (32 KB)
+constexpr int kMaxLocalFloats = 8192;              // slopes of a block's slices (32 KB), as slope_floats pads them
 constexpr int kMaxRowFloats = 4096;                // rows a block reduces, at most
 constexpr size_t kDynSmemBudget = 227 * 1024 - 2048;  // dynamic shared memory per block
 // The per-frame kernels leave room on their SM for a block of the sum kernel
@@ -1372,11 +1372,14 @@ using Launch = LaunchPlan;
 // Measured, loop (host to host) and frame after frame, INT8, tensor cores -> chains:
 // 8x8 12.6 -> 11.4 and 6.5 -> 5.6 us, 26x26 (8 columns x 2 rows) 12.8 -> 12.4 and 6.1 ->
 // 5.4, 34x34 (12 x 3) 13.1 -> 12.7 and 6.4 -> 6.0; beyond the line FP16 41x41 (18 x 4)
-// 13.7 -> 14.0 and 6.9 -> 7.4.  Every slice of a matrix goes the same way, in all kernels.
-constexpr int kChainSteps = 40;
+// 13.7 -> 14.0 and 6.9 -> 7.4, FP8 frames 6.8 -> 7.2.  INT8 converts more cheaply and has
+// its line higher: 41x41 of 7 px 15.1 -> 14.7 and 7.0 -> 7.0.  Every slice of a matrix goes
+// the same way, in all kernels.
+constexpr int kChainSteps = 40, kChainStepsInt8 = 90;
 template <int DT> struct CanChain { static constexpr bool v = DT != RTC_F32; };
-inline bool chain_rule(int max_rb, int esz, int nact) {
-    return esz < 4 && max_rb / esz * static_cast<long long>((nact + kConsumers - 1) / kConsumers) <= kChainSteps;
+inline bool chain_rule(int max_rb, int store, int esz, int nact) {
+    const int steps = store == RTC_INT8 ? kChainStepsInt8 : kChainSteps;
+    return esz < 4 && max_rb / esz * static_cast<long long>((nact + kConsumers - 1) / kConsumers) <= steps;
 }
 constexpr int kNoPredecessor = -1;
 
@@ -1390,7 +1393,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     L.G = S < h->num_sms ? S : h->num_sms;
     if (L.G < 1 || S < 1 || static_cast<int>(h->sl_rowbytes.size()) != S) return L;
     // largest row and largest block-local slope vector over the blocks
-    int max_rb = 0, max_loc = 0;
+    int max_rb = 0, max_loc = 0, max_floats = 0;
     const bool frag = h->sl_frag;
     const int esz = h->sl_esz;
     for (int b = 0; b < L.G; ++b) {
@@ -1408,7 +1411,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
     L.loc_floats = (max_loc + 3) / 4 * 4;
     L.row_floats = (h->cfg.nact + L.G - 1) / L.G;
     L.region = (min_region + 15) / 16 * 16;
-    L.chain = chain_rule(max_rb, esz, h->cfg.nact);
+    L.chain = chain_rule(max_rb, h->store, esz, h->cfg.nact);
     L.bf_floats = frag ? bfrag_floats(L.loc_floats) : 0;
     const size_t slopes = 4 * static_cast<size_t>(L.loc_floats + L.bf_floats + (frag ? L.max_slices : 0));
     size_t extra = L.region + slopes + 8 * static_cast<size_t>(L.row_floats) + 4 * kConsumerWarps * 32;
@@ -1448,7 +1451,7 @@ inline Launch plan_launch(const rtc_handle* h, size_t min_region = 0, bool loop 
         L.pre_tiles = most ? 0 : 1;
         L.l2_ahead = most ? 0 : 1;
     }
-    L.ok = L.nst >= 2 && L.loc_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
+    L.ok = L.nst >= 2 && max_floats <= kMaxLocalFloats && L.row_floats <= kMaxRowFloats &&
            S <= kMaxSlices && L.smem <= budget;
     if (frag) L.T = 1;
     return L;
