@@ -85,7 +85,7 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
-    pdl_launch_dependents();
+    if (!g.late) pdl_launch_dependents();
     const Plan pl = make_plan(g, smem);
     // the grid position of a consumer's first subaperture, loaded before the
     // block's set-up so that its latency overlaps it
@@ -103,6 +103,7 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     pdl_wait();                         // before the partials of the last frame are overwritten
     consumer_sync();
     consume<DT, CHAIN>(g, pl, sh, tid, 0);
+    if (g.late) pdl_launch_dependents();
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
@@ -131,7 +132,7 @@ frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned*
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
-    pdl_launch_dependents();
+    if (!g.late) pdl_launch_dependents();
     const Plan pl = make_plan(g, smem);
     if (tid == 0) init_shared(sh);
     __syncthreads();
@@ -155,6 +156,7 @@ frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned*
         });
     consumer_sync();
     consume<DT, CHAIN>(g, pl, sh, tid, 0);
+    if (g.late) pdl_launch_dependents();
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);

@@ -253,6 +253,15 @@ int take_status(rtc_handle* h, cudaStream_t st) {
     return RTC_OK;
 }
 
+const void* mapped_view(const void* p) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();             // clear the error of a pointer CUDA does not know
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+}
+
 namespace {
 
 int check_ready(rtc_handle* h) {
@@ -327,16 +336,6 @@ int enqueue_step(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float*
     return RTC_OK;
 }
 
-// Device view of a pinned, mapped host buffer; nullptr for pageable or device memory.
-const void* mapped_view(const void* p) {
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();             // clear the error of a pointer CUDA does not know
-        return nullptr;
-    }
-    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
-}
-void* mapped_view(void* p) { return const_cast<void*>(mapped_view(static_cast<const void*>(p))); }
 
 constexpr double kHostWaitS = 2.0;      // bound on the host's wait for a frame's record
 

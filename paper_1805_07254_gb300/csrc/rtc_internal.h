@@ -165,6 +165,10 @@ struct rtc_handle {
     std::string err;
 };
 
+// Device view of a pinned, mapped host buffer; nullptr for pageable or device memory.
+const void* mapped_view(const void* p);
+inline void* mapped_view(void* p) { return const_cast<void*>(mapped_view(static_cast<const void*>(p))); }
+
 // Pixel calibration + centre of gravity + slope packing for every valid
 // subaperture of every WFS frame.  Writes s[0 .. nslopes) and, unless null, s2.  early:
 // the next kernel of the stream is one that reads nothing before its wait that a kernel
