@@ -154,7 +154,9 @@ struct rtc_handle {
     float* d_ring = nullptr;                  // [4][kpad] last measured slope vectors
     int ring_head = 3;                        // row of the newest vector
     float* d_spred = nullptr;                 // [kpad] predicted slopes, zero padded
-    int* h_status = nullptr;        // pinned host mirror of d_status
+    int* h_status = nullptr;        // pinned host mirror of d_status, and behind it
+    float* h_dm = nullptr;          // [nact] DM commands of a frame whose caller's buffer is pageable,
+    float* d_hdm = nullptr;         // and their device view
     // rtc_process_frame with pinned host buffers (allocated at its first such call)
     rtc_pf_done* h_pf_done = nullptr;         // pinned mapped completion record
     rtc_pf_done* d_pf_done = nullptr;         // its device view
@@ -165,6 +167,8 @@ struct rtc_handle {
     std::string err;
 };
 
+// Whether p is memory that the host can write by itself (pageable or pinned).
+bool host_memory(const void* p);
 // Device view of a pinned, mapped host buffer; nullptr for pageable or device memory.
 const void* mapped_view(const void* p);
 inline void* mapped_view(void* p) { return const_cast<void*>(mapped_view(static_cast<const void*>(p))); }

@@ -108,3 +108,20 @@ def test_only_the_marked_step_is_left_out(poke, nsub, nact, store, host):
     b.reconstruct_async(None, ref, stream=st)
     torch.cuda.synchronize()
     assert torch.equal(dm, ref)
+
+
+def test_pageable_frame_reports_the_kept_state(poke):
+    """A synchronous frame from pageable memory whose wait expired raises, its dm_out holds
+    the state that was kept, and the next frame goes on from there."""
+    from paper_1805_07254_gb300.rtc import RtcError
+    a, b, frames = _pair(24, 460, "f32", False)
+    f = frames.cpu().numpy()[:, None]
+    first = a.process_frame(f[0])
+    assert np.array_equal(first, b.process_frame(f[0]))
+    poke(a, 0)
+    poke(a, 1)
+    out = np.full(460, 7.0, np.float32)
+    with pytest.raises(RtcError):
+        a.process_frame(f[1], dm_out=out)
+    assert np.array_equal(out, first)
+    assert np.array_equal(a.process_frame(f[2]), b.process_frame(f[2]))
