@@ -540,7 +540,8 @@ __global__ void __launch_bounds__(256) mlp_update_kernel(MlpDev w, const float* 
     // the step's own state: last written by the update before the train kernel that
     // this launch depends on, which waited for it before it let this one start
     const bool own = tid < kUpdateParams && p < NPARAM && lr > 0.f;
-    const float m0 = own ? w.m[p] : 0.f, v0 = own ? w.v[p] : 0.f, w0 = own ? w.master[p] : 0.f;
+    const float m0 = own ? __ldcg(w.m + p) : 0.f, v0 = own ? __ldcg(w.v + p) : 0.f;   // (never from a stale L1)
+    const float w0 = own ? __ldcg(w.master + p) : 0.f;
     pdl_wait();
     pdl_launch_dependents();
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
