@@ -85,6 +85,7 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
     const Plan pl = make_plan(g, smem);
     // the grid position of a consumer's first subaperture, loaded before the
     // block's set-up so that its latency overlaps it
@@ -92,7 +93,6 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     const int2 pos0 = rtc_pixel::subap_pos(px, pl.g0 + slot, tid < kConsumers && pl.g0 + slot < pl.g1);
     if (tid == 0) init_shared(sh);
     __syncthreads();
-    if (!g.late) pdl_launch_dependents();   // (as the first instruction it waited for the parameter)
     if (tid >= kConsumers) {
         if ((tid & 31) == 0) produce(g, pl, sh);
         return;
@@ -103,7 +103,6 @@ frame_kernel(rtc_pixel::PixelArgs px, Args g, FrameHost fh, SumArgs sa, unsigned
     pdl_wait();                         // before the partials of the last frame are overwritten
     consumer_sync();
     consume<DT, CHAIN>(g, pl, sh, tid, 0);
-    if (g.late) pdl_launch_dependents();
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);
@@ -132,10 +131,10 @@ frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned*
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ Shared sh;
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
     const Plan pl = make_plan(g, smem);
     if (tid == 0) init_shared(sh);
     __syncthreads();
-    if (!g.late) pdl_launch_dependents();   // (as the first instruction it waited for the parameter)
     if (tid >= kConsumers) {
         if ((tid & 31) == 0) produce(g, pl, sh);
         return;
@@ -156,7 +155,6 @@ frame_pred_kernel(Args g, rtc_pred::PredArgs pa, int head, SumArgs sa, unsigned*
         });
     consumer_sync();
     consume<DT, CHAIN>(g, pl, sh, tid, 0);
-    if (g.late) pdl_launch_dependents();
     if (LAST) {
         __shared__ int last;
         last_block_sum(sa, ctr, reinterpret_cast<float*>(smem), &last, tid);

@@ -8,10 +8,7 @@
 // launches need not be cooperative ones, which start only on an idle device.  Both are
 // launched with programmatic dependent launch and let their successor start at once:
 //   - the sum's blocks are small enough to sit on the SMs beside the streaming blocks
-//     and wait there, in hardware, for the partials (in a server slot they start when the
-//     stream is done: the SMs have room for the waiting blocks of one job, and those of
-//     another would queue up behind them; four ELT FP32 jobs 30.1 -> 28.3 us a frame, BF16
-//     22.7 -> 22.1);
+//     and wait there, in hardware, for the partials;
 //   - the next frame's streaming blocks start as soon as this frame's leave their SM:
 //     their set-up and the fill of the ring (30 MB of the next matrix stream) run during
 //     the slowest blocks, the sum, and the hand-over, and they wait only before they
@@ -86,7 +83,12 @@ __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, Fr
     }
     red[warp * 32 + lane] = v;
     __syncthreads();
-    if (tid == 0 && cut != RTC_OK && atomicInc(r.cutctr, gridDim.x - 1) == gridDim.x - 1) *r.cut = RTC_OK;
+    // (here: with it at the kernel's end frames one after another took up to 0.4 us more,
+    // and frames from the host, here, 0.2 us)
+    auto clear = [&]() {
+        if (tid == 0 && cut != RTC_OK && atomicInc(r.cutctr, gridDim.x - 1) == gridDim.x - 1) *r.cut = RTC_OK;
+    };
+    if (!HOST) clear();
     if (mine && cut == RTC_OK) {
         float t[kConsumerWarps];
 #pragma unroll
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(kConsumers, 4) mvm_reduce_kernel(SumArgs r, Fr
         r.a[row] = an;
         if (r.dm_out) r.dm_out[row] = an;
     }
+    if (HOST) clear();
     if (HOST) {
         __syncthreads();
         if (tid == 0) finish_host(fh, r.status);
@@ -149,7 +152,15 @@ rtc_mvm::SumArgs sum_args(const rtc_handle* h, float* d_dm_out) {
 cudaError_t launch_sum(rtc_handle* h, float* d_dm_out, cudaStream_t st, FrameHost* fh) {
     const SumArgs r = sum_args(h, d_dm_out);
     const dim3 grid((h->cfg.nact + 31) / 32), block(kConsumers);
-    if (!fh) return launch_pdl(mvm_reduce_kernel<false>, grid, block, 0, st, r, FrameHost{});
+    if (!fh) {
+        // In a server slot with a matrix that comes from the HBM every frame, the sum starts
+        // when the stream is done: the SMs have room for one job's waiting blocks beside
+        // the streaming ones, and those of other jobs would queue up behind them for the
+        // whole of its long stream (four ELT FP32 jobs 30.2 us a frame, so 28.4).  Other
+        // slots gain from the early start (eight 41x41 FP16 jobs 12.9 against 13.7).
+        const bool overlap = !h->in_slot || h->m_bytes <= kL2KeepBytes;
+        return launch_pdl_if(overlap, mvm_reduce_kernel<false>, grid, block, 0, st, r, FrameHost{});
+    }
     fh->target = h->pf_arrivals + grid.x;
     const cudaError_t e = launch_pdl(mvm_reduce_kernel<true>, grid, block, 0, st, r, *fh);
     if (e == cudaSuccess) h->pf_arrivals = fh->target;

@@ -329,7 +329,6 @@ struct Args {
     float gain, leak;
     int* status;             // device error word, kept until the host reads it
     int* cut;                // mark of this launch alone (see record_timeout)
-    int late;                // let the sum start after the stream, not at once (server slots)
 };
 
 struct Shared {
@@ -1498,7 +1497,6 @@ inline Args make_args(const rtc_handle* h, const float* d_s, const Launch& L) {
     g.leak = h->leak;
     g.status = h->d_status;
     g.cut = h->d_status + 1;
-    g.late = h->in_slot ? 1 : 0;
     return g;
 }
 
