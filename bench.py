@@ -243,7 +243,7 @@ def workload_config(cfg, store, info=None, predictor=False):
 def time_steps(torch, r, d_frames, d_dm, flush, st, n_steps, n_warm, fused=True):
     """Per-step device times (us) from CUDA events on stream st.
 
-    fused: one rtc_process_frame_async call per step (the fused frame kernel);
+    fused: one rtc_process_frame_async call per step (a frame's kernels);
     returns (step,).  Otherwise the two stage calls with an event between them;
     returns (pixel stage, reconstruction, step)."""
     E = torch.cuda.Event
@@ -311,9 +311,10 @@ def launch_floor(torch, flush, st, n_steps, n_warm=20):
 
 def e2e_entry(s_launch, s_res, resident_headline, info, cfg, n, step_in_bytes, l2_bytes):
     """The e2e object: rtc_process_frame with pinned host buffers, synchronous, host
-    clock.  Two modes of the same call: one kernel launch per call (L2 flushed before
-    each call) and the resident kernel (rtc_resident_start; no flush possible).  The
-    resident figure is the headline when the step's inputs exceed L2."""
+    clock.  Two modes of the same call: the call's own kernel launches (L2 flushed
+    before each call) and the resident kernel (rtc_resident_start; no flush possible).  The
+    resident figure is the headline when the step's inputs exceed L2.  (The mode's label
+    is older than the second kernel of a frame; readers of the line know it by that.)"""
     launch = {"p50_us": round(s_launch["p50"], 3), "p99_us": round(s_launch["p99"], 3),
               "rms_jitter_us": round(s_launch["rms_jitter"], 3), "l2": "flushed before each call"}
     res = {"p50_us": round(s_res["p50"], 3), "p99_us": round(s_res["p99"], 3),
@@ -488,8 +489,8 @@ def ours(args):
             rv.close()
 
     # reduced precision + learned predictor: BF16 matrix, predictor on (pixel stage,
-    # prediction and streaming reconstruction in one launch); the weights do not
-    # change the timing
+    # prediction with the streaming reconstruction, and the sum: three kernels); the
+    # weights do not change the timing
     if not args.no_variants:
         rp = controller("bf16")
         rp.load_predictor(pred_params, 0.3)

@@ -171,7 +171,10 @@ int rtc_process_frame(rtc_handle* h, const uint16_t* frame, float* dm_out, float
  * work) without synchronising.  d_frame must be 16-byte
  * aligned.  d_dm_out (float32 [nact]) and d_slopes_out (float32 [nslopes]) may
  * be NULL.  The integrator state lives on the device; consecutive calls on one
- * stream form the closed loop.  Errors: RTC_EINVAL, RTC_ESTATE, RTC_EDEVICE. */
+ * stream form the closed loop.  Every wait of a kernel for its own copies is bounded
+ * (200 ms): a call in which one expires leaves the integrator and d_dm_out as they
+ * were, the calls after it run as usual, and rtc_synchronize reports RTC_ETIMEDOUT.
+ * Errors: RTC_EINVAL, RTC_ESTATE, RTC_EDEVICE. */
 int rtc_process_frame_async(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out,
                             float* d_slopes_out, void* stream);
 
@@ -363,7 +366,7 @@ int rtc_server_destroy(rtc_server* s);
 
 /* Admit a job: frames host uint16 [n_frames][n_wfs][H][W] (pinned memory keeps the
  * submission asynchronous), dm_out host float32 [n_frames][nact] receives each
- * frame's DM commands.  Both stay owned by the caller and must stay valid until
+ * frame's DM commands (written by the job's kernels if it is pinned).  Both stay owned by the caller and must stay valid until
  * rtc_slot_poll reports the job done; meanwhile the handle's own calls (rtc_destroy
  * included) return RTC_ESTATE, since the job's kernels use its device state.
  * *slot receives the slot id.  Errors: RTC_EINVAL, RTC_ESTATE (handle not ready
@@ -451,9 +454,10 @@ int rtc_mlp_predict_seq(rtc_mlp* m, const float* d_S, int32_t n_frames, float si
  * the features.  The handle keeps the last 4 measured slope vectors; with the
  * predictor on, the reconstruction uses the predicted next slopes
  * s_k + sigma * y instead of the measured ones, in rtc_process_frame(_async) and
- * in rtc_run_loop alike (the prediction runs inside the same kernel launch as the
- * rest of the frame), and slopes_out still receives the measured slopes.
- * rtc_reset clears the history.  Errors: RTC_EINVAL, RTC_ENOMEM, RTC_EDEVICE. */
+ * in rtc_run_loop alike, and slopes_out still receives the measured slopes.
+ * rtc_reset clears the history.  (In the loop the prediction runs inside the persistent
+ * kernel; a per-frame call is three launches with it and two without, one fewer for
+ * small systems.)  Errors: RTC_EINVAL, RTC_ENOMEM, RTC_EDEVICE. */
 int rtc_load_predictor(rtc_handle* h, const float* params, int64_t n, float sigma);
 int rtc_set_predictor(rtc_handle* h, int32_t on);
 

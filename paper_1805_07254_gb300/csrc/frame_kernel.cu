@@ -8,9 +8,9 @@
 // consumer warps compute the block's slopes (pixel.cuh) into shared memory and
 // multiply them straight away: no block waits for another, as in the paper's
 // per-thread column blocks (Sec. 2.3).  Each block writes one partial DM vector per
-// slice.  The producer starts at once, before the previous kernel of the stream has
-// finished, and so do the subaperture positions and the calibration data; the block
-// waits for its predecessor before it reads pixels.
+// slice.  The block's set-up, the subaperture positions, the calibration data and, as
+// plan_launch says, the first matrix tiles come before the previous kernel of the stream
+// has finished; the block waits for it before it reads pixels.
 //
 // With the learned slope predictor on, the measured slopes of all blocks have to be
 // known before any can predict, so the pixel stage is a kernel of its own: it writes
@@ -28,11 +28,10 @@
 // except for HOST frames.
 //
 // Measured, frame after frame on one stream (one cooperative kernel with a grid barrier
-// -> this): ELT FP32 28.9 -> 23.1 us, INT8 20.9 -> 12.9, BF16 with prediction 28.4 ->
-// 24.6, six ELT sensors FP8 59.4 -> 47.4, 41x41 FP16 12.3 -> 7.9 of GPU time (9.2 with
-// the two launches' host time, which bounds it) and 8x8 FP32 10.3 -> 6.8.  Of an FP32
-// frame the blocks stream 17 us (6.5 TB/s); slopes are known 2.9 us after the last
-// frame's sum, the hand-over to the sum takes 0.9 us and the sum 1.4.
+// -> this): ELT FP32 28.8 -> 22.8 us (its bytes need 21.3), INT8 20.9 -> 13.0, BF16 with
+// prediction 28.3 -> 24.1, six ELT sensors FP8 59.4 -> 48.0, 41x41 FP16 12.3 -> 6.8 of GPU
+// time (8.8 with the two launches' host time, which bounds it) and 8x8 FP32 12.3 -> 6.1
+// (7.2).
 
 #include "launch.cuh"
 #include "mlp.h"

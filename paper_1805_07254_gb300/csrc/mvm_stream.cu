@@ -10,9 +10,9 @@
 //   - the sum's blocks are small enough to sit on the SMs beside the streaming blocks
 //     and wait there, in hardware, for the partials;
 //   - the next frame's streaming blocks start as soon as this frame's leave their SM:
-//     their set-up and the fill of the ring (30 MB of the next matrix stream) run during
-//     the slowest blocks, the sum, and the hand-over, and they wait only before they
-//     read pixels.
+//     their set-up and their first matrix tiles (none or one for most frames, the whole
+//     ring for some: plan_launch, stream_mvm.cuh) run during the slowest blocks, the sum,
+//     and the hand-over, and they wait only before they read pixels.
 // Everything a kernel reads before its wait is written by no kernel (matrix, slice
 // table, maps, row scales).  frame_kernel.cu has the figures of this and of one
 // cooperative kernel with a grid barrier, whose launch waited for an idle device.

@@ -1,7 +1,7 @@
 // Fused inference of the learned slope predictor (the network of mlp.cu) for one
-// block's share of the subapertures, run by the consumer warps of the frame and
-// loop kernels between their two grid barriers:
-//   pixel stage -> grid barrier -> predict (this file) -> grid barrier -> MVM.
+// block's share of the subapertures, run by the consumer warps of frame_pred_kernel,
+// after the pixel kernel, and of the loop kernel, after the grid barrier that follows
+// its pixel stage; the block then multiplies the predicted slopes.
 //
 // The network is small (200 -> 64 -> 64 -> 2), so the phase is latency-bound:
 // the BF16 weight fragments of both hidden layers, their biases and the
@@ -178,8 +178,9 @@ __device__ __forceinline__ int pair_nbr(const PredArgs& pa, int t0, int i1, int 
 // features of the three older frames (ring rows head-1 .. head-3, written by earlier
 // frames) in registers, and the output layer's weights in the scratch sm
 // (asynchronous copies, complete once predict's first barrier has passed).
-// [i0, i1): the block's subapertures.  Call it after the block's grid-barrier
-// arrival (a release would wait for these loads) and before its wait.  OLDER = false
+// [i0, i1): the block's subapertures.  Called before the wait for the measured slopes: in
+// the loop after the block's grid-barrier arrival (a release would wait for these
+// loads), in frame_pred_kernel before the wait for the pixel kernel.  OLDER = false
 // leaves the older frames' features to predict: a kernel that may start before the
 // kernels that wrote those rows are known to be complete.
 template <bool OLDER>
@@ -221,10 +222,10 @@ __device__ __forceinline__ void prefetch(const PredArgs& pa, unsigned char* sm, 
         }
 }
 
-// After the grid barrier that completes the measured slopes: predictions of
+// Once the measured slopes are complete: predictions of
 // subapertures [i0, i1) from the ring rows head, head-1, head-2, head-3 (newest
-// first), with the registers and scratch `prefetch` filled (before the barrier, so
-// that the weight and neighbour loads overlap the wait).  Every consumer thread
+// first), with the registers and scratch `prefetch` filled (before the wait, so
+// that the weight and neighbour loads overlap it).  Every consumer thread
 // calls it; sm is TS-sample scratch of kSmemBytes.  src(i, axis) gives the block's
 // own copy of the measured slope s_k of subaperture i (the value in ring row head);
 // each prediction goes to pa.s_pred and to sink(i, axis, value), after the same

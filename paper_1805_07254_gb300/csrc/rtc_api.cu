@@ -106,8 +106,8 @@ std::vector<int> slice_bounds(const rtc_handle* h, int esz) {
 // The slice table for slice bounds g0, in the handle's host vectors: each slice one
 // contiguous [nact][2 n_s] block (x slopes, then y slopes): FP32 rows padded until an
 // access unit (16, 8 or 4 bytes) divides them an odd number of times, 1- and 2-byte
-// stores unpadded in fragment order (rtc_mvm::slice_elem_offset).  colmap: column c (WFS w, axis, subaperture i) -> (slice,
-// column within the slice).
+// stores unpadded in fragment order (rtc_mvm::slice_elem_offset).  colmap: column c (WFS
+// w, axis, subaperture i) -> (slice, column within the slice).
 void cut_slices(rtc_handle* h, const std::vector<int>& g0, int esz, std::vector<int2>& colmap) {
     const int S = static_cast<int>(g0.size()) - 1;
     const int nact = h->cfg.nact;
@@ -243,7 +243,7 @@ int take_status(rtc_handle* h, cudaStream_t st) {
     RTC_CUDA(h, cudaStreamSynchronize(st));
     const int code = *h->h_status;
     if (code != 0) {
-        // an aborted launch may leave the grid-barrier count short: start it afresh
+        // an aborted loop may leave the grid-barrier count short: start it afresh
         RTC_CUDA(h, cudaMemsetAsync(h->d_gridbar, 0, sizeof(unsigned long long), st));
         h->grid_epoch = 0;
         RTC_CUDA(h, cudaMemsetAsync(h->d_status, 0, 2 * sizeof(int), st));
@@ -327,7 +327,7 @@ int enqueue_step(rtc_handle* h, const uint16_t* d_frame, float* d_dm_out, float*
     float* direct = d_slopes_out && h->kpad > 0 && slopes_direct(h, d_slopes_out, d_frame, d_dm_out) ? d_slopes_out : nullptr;
     if (h->pred_on && h->kpad > 0) {
         // measured slopes into the next row of the history ring, the prediction from
-        // the 4 newest rows, the reconstruction from the prediction: one launch
+        // the 4 newest rows, the reconstruction from the prediction
         const int head = (h->ring_head + 1) & 3;
         float* s_meas = h->d_ring + static_cast<size_t>(head) * h->kpad;
         RTC_CUDA(h, launch_frame(h, d_frame, d_dm_out, s_meas, head, st, fh, direct));
@@ -360,8 +360,8 @@ long long g_host_stamps[5];
     } while (0)
 #endif
 
-// rtc_process_frame on pinned host buffers: one launch reads the frame over the host
-// link and writes the DM commands there; the host waits for the completion record.
+// rtc_process_frame on pinned host buffers: the kernels read the frame over the host
+// link and write the DM commands there; the host waits for the completion record.
 int process_mapped(rtc_handle* h, const uint16_t* d_frame_host, float* d_dm_host, float* slopes_out) {
     if (!h->h_pf_done) {
         void* p = nullptr;

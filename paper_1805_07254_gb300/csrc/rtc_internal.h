@@ -23,7 +23,7 @@ struct rtc_loop_done {
 };
 
 // Completion record of one rtc_process_frame call whose buffers are in pinned host
-// memory, written by the last block of the frame kernel into mapped host memory.
+// memory, written by the last block of the sum kernel into mapped host memory.
 struct rtc_pf_done {
     unsigned long long seq;      // the call's sequence number once its DM commands are written
     int status;                  // the device status word at that time (RTC_OK or an error)

@@ -30,8 +30,9 @@
 // (rows are padded until one does), so that the rows a warp reads at once fall in
 // different banks; all lanes read the same units of the slice's slopes at the same
 // time (shared-memory broadcasts).  1- and 2-byte stores go to the tensor cores, 16 rows
-// an instruction, the slopes split into parts (see make_bfrag); the FP8 and INT8 row
-// scales are applied once per row after the sum over slices.
+// an instruction, the slopes split into parts (see make_bfrag), or, where slices are
+// small (chain_rule) or a slope does not split exactly (wide_slices), through FP32 FMAs;
+// the FP8 and INT8 row scales are applied once per row after the sum over slices.
 //
 // Every wait is bounded (200 ms of %globaltimer); a wait that expires records
 // RTC_ETIMEDOUT in the status word, the block skips the rest of its work, lets its
@@ -1364,6 +1365,9 @@ __device__ __forceinline__ void finish_host(const FrameHost& fh, const int* stat
 //   - several pixel rounds a block (more sensors): the ring early and nothing ahead,
 //     the pixel stage itself takes the HBM (six sensors FP8 47.8 us against 50).
 //     Prediction frames too, whose blocks have the whole pixel kernel to wait for.
+// (Against one cooperative kernel a frame every system between 8x8 and 74x74, with one to
+// six sensors and every store, is faster under these rules, one frame after another and
+// alone with cold caches.)
 using Launch = LaunchPlan;
 
 // Small slices of 1- and 2-byte stores: FP32 chains instead of the tensor cores.  Splitting
